@@ -239,6 +239,12 @@ __device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, un
     return d;
 }
 
+__device__ __forceinline__ unsigned long long mul_f32x2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // Transpose of an 8 x 8 matrix of 16-bit elements held two per lane (lane t:
 // row t / 4, columns 2 (t % 4) and 2 (t % 4) + 1): lane t gets the same
 // positions of the transpose.

@@ -81,7 +81,12 @@ constexpr int64_t kSpareEntriesNum = 3, kSpareEntriesDen = 2;
 // 842.8 -> 839.4 us; the two-level tree (2/3 of its tile-pages in pieces of
 // two or more tiles) 77.6 -> 87.8 us, so it stays on single tiles.
 constexpr int64_t kPairShareNum = 3, kPairShareDen = 4;
+// fp32 pieces: one CTA each, 3 CTAs per SM.  About kFp32Waves pieces per CTA
+// slot even out the launch's end; never longer than kFp32ChunkPages (the
+// fixed length before: 2 to 3 pieces a slot on a 16-branch step).
 constexpr int kFp32ChunkPages = 32;
+constexpr int kFp32MinPages = 4;
+constexpr int64_t kFp32Slots = 3, kFp32Waves = 3;
 // stream rows kept free after a branch's last item: half its pages, 4 to 64
 // (an item that grows further makes the launch's tail: build a new plan)
 constexpr int32_t kAppendSlackMin = 4, kAppendSlackMax = 64;
@@ -720,8 +725,24 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
         return true;
     };
     if (mode == PARASON_FP32) {
+        int64_t pages = 0;
+        for (const Run &r : runs) pages += r.pages;
+        int64_t chunk = std::min<int64_t>(
+            kFp32ChunkPages,
+            std::max<int64_t>(kFp32MinPages, pages / (kFp32Slots * kFp32Waves * p->num_sms)));
+        // shorter pieces mean more partial rows: not past what a decode
+        // without a caller's workspace holds
+        int64_t rows = 0;
+        for (const Run &r : runs) {
+            int64_t per = 0, n = 0;
+            piece_split(r.pages, chunk, 1, per, n);
+            rows += n * r.nrows;
+        }
+        const int64_t row_bytes = static_cast<int64_t>(cfg->head_dim) * 4 + 8;
+        if (rows * row_bytes + 2 * static_cast<int64_t>(kAlign) > PARASON_NO_ALLOC_SCRATCH_BYTES)
+            chunk = kFp32ChunkPages;
         for (const Run &r : runs)
-            if (!cut(r, kFp32ChunkPages, 1)) return PARASON_EUNSUPPORTED;
+            if (!cut(r, chunk, 1)) return PARASON_EUNSUPPORTED;
     } else {
         const int64_t total_warps = static_cast<int64_t>(p->num_sms) * p->suffix_warps;
         const int64_t narrow_chunk = std::min<int64_t>(
@@ -1507,10 +1528,9 @@ parason_status parason_attn_decode(parason_plan p, const void *q, const void *k_
     m.queue_next = p->d_queue_next;
     m.queue_start[0] = p->queue_start[0];
     m.queue_start[1] = p->queue_start[1];
-    // programmatic dependent launch after the persistent kernel: the merge
+    // programmatic dependent launch after the attention kernel: the merge
     // grid is launched while the attention grid drains, and waits for it
-    const bool pdl = has_items && p->cfg.mode != PARASON_FP32;
-    if (parason::launch_merge(m, d, p->cfg.mode, pdl, stream) != cudaSuccess) return PARASON_ECUDA;
+    if (parason::launch_merge(m, d, p->cfg.mode, has_items, stream) != cudaSuccess) return PARASON_ECUDA;
     st = record_event(p, 2, stream);
     if (st != PARASON_OK) return st;
     if (p->timing_cap > 0 && p->timing_n < p->timing_cap) p->timing_n++;
