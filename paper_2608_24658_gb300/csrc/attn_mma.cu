@@ -14,7 +14,7 @@
 //        producer warp moves 64-token blocks of K and V by TMA (one 5-D box
 //        per column block when the block's 4 pages are consecutive in the
 //        pool, else 3-D boxes per page) into a 6-stage ring (with e4m3 KV,
-//        4 raw stages and 4 converted ones); one thread issues S = Q K^T and
+//        4 raw stages and 4 converted ones); one warp issues S = Q K^T and
 //        another O += P V as tcgen05.mma with Q, S/P and O in TMEM and K, V
 //        from shared memory; 4 softmax warps own one row per thread (TMEM
 //        lane) and write P over S; 4 epilogue warps store an item's O and
@@ -1176,10 +1176,10 @@ __device__ void prefix_cta(const CUtensorMap *tmap_k, const CUtensorMap *tmap_v,
 //               consecutive in the pool (the 5-D run maps), else one per
 //               page and column block; pages past the item's end are loaded
 //               from an out-of-range row, which TMA fills with zeros
-//   warp 9      S issuer (one thread): S = Q K^T (M 128, N 64, K 128) into
+//   warp 9      S issuer (one lane): S = Q K^T (M 128, N 64, K 128) into
 //               one of two TMEM buffers, once PV of the block two back has
 //               freed it; runs ahead across item boundaries
-//   warp 11     PV issuer (one thread): O += P V (M 128, N 128, K 64) into
+//   warp 11     PV issuer (one lane): O += P V (M 128, N 128, K 64) into
 //               the item's TMEM accumulator (two, alternating by item).
 //               A (Q or P) comes from TMEM, B (K or V) from shared memory.
 //               tcgen05.commit releases ring stages and signals completion.
@@ -1548,60 +1548,62 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                                            kDrainLimitNs, nullptr);
     } else if (warp == kTcMmaWarp || warp == kTcPvWarp) {
         // ------------------------------------------------------------ MMA issuers
-        if (lane == 0) {
-            // Two threads issue, so that neither product waits behind the other's
-            // issue (an MMA takes about 45 cycles to issue; twelve per block on
-            // one thread held the tile back).  Warp 9 issues S = Q K^T of every
-            // block, warp 11 O += P V.  S(b) overwrites the buffer of P(b - 2),
-            // so it waits for PV(b - 2) to complete.
+        {
+            // Two warps issue, so that neither product waits behind the other's
+            // issue; in each the whole warp runs the loop and one elected lane
+            // issues (see elect_one).  Warp 9 issues S = Q K^T of every block,
+            // warp 11 O += P V.  S(b) overwrites the buffer of P(b - 2), so it
+            // waits for PV(b - 2) to complete.
             constexpr uint32_t kIdS = kF8 ? tc::idesc_f16_f32(kTcRows, kTcBlockTokens, false)
                                           : tc::idesc_bf16_f32(kTcRows, kTcBlockTokens, false);
             constexpr uint32_t kIdPV = kF8 ? tc::idesc_f16_f32(kTcRows, D, true)
                                            : tc::idesc_bf16_f32(kTcRows, D, true);
             constexpr int kMmaStages = kF8 ? kTcCvStages : kTcStages;
+            // A wait that runs out leaves its mark, and the warp goes on together
+            // to the next point where it looks (lanes that part would leave the
+            // others waiting in elect.sync; what is issued in between works on
+            // this CTA's own memory and is thrown away).
+            bool bad = false;
             auto wait = [&](int i, int parity) {
-                return tc_wait(bar(i), static_cast<uint32_t>(parity & 1), limit, abort_flag);
+                if (!tc_wait(bar(i), static_cast<uint32_t>(parity & 1), limit, abort_flag)) {
+                    tc_fail(a, abort_flag, kSiteConsumerFull);
+                    bad = true;
+                }
             };
+            auto failed = [&]() { return __any_sync(0xffffffffu, bad) != 0; };
             // descriptors of stage 0; a stage, a column block or a K step moves
             // the start address field (address / 16) by a constant
             const uint32_t mma_ring = kF8 ? ring + kTcCvOffset : ring;
             const uint64_t desc_k = tc::smem_desc_sw128(mma_ring, 16, 1024);
             const uint64_t desc_v = tc::smem_desc_sw128(mma_ring + kTcKBytes, kTcColBlockBytes, 1024);
             constexpr uint32_t kStageStep = kTcStageBytes >> 4;
-            bool ok = true;
             int b = 0;                       // block of the CTA's stream
             int st = 0, ph = 0;              // its stage and the stage's phase parity
-            for (int k = 0; ok; ++k) {
+            for (int k = 0;; ++k) {
                 const int ms = k % kTcMeta;
-                if (!wait(kBarMetaFull + ms, k / kTcMeta)) {
-                    ok = false;
-                    break;
-                }
-                if (meta[ms].id < 0) break;
+                wait(kBarMetaFull + ms, k / kTcMeta);
+                if (failed() || meta[ms].id < 0) break;
                 const int nb = tc_blocks(meta[ms].it.num_pages);
                 if (warp == kTcMmaWarp) {
                     // S of the item's blocks, with its Q (buffer k & 1)
-                    if (!wait(kBarQReady + (k & 1), k >> 1)) {
-                        ok = false;
-                        break;
-                    }
+                    wait(kBarQReady + (k & 1), k >> 1);
                     const uint32_t tQ = tmem + kTmemQ + 64u * (k & 1);
                     for (int i = 0; i < nb; ++i, ++b) {
-                        if (!wait((kF8 ? kBarCvFull : kBarKvFull) + st, ph) ||
-                            (b >= 2 && !wait(kBarPvDone + (b & 1), (b - 2) >> 1))) {
-                            ok = false;
-                            break;
-                        }
+                        if (failed()) break;
+                        wait((kF8 ? kBarCvFull : kBarKvFull) + st, ph);
+                        if (b >= 2) wait(kBarPvDone + (b & 1), (b - 2) >> 1);
                         tc::fence_after_sync();
                         const uint32_t tS = tmem + kTmemS + 64u * (b & 1);
                         const uint64_t kd = desc_k + static_cast<uint64_t>(st * kStageStep);
+                        if (tc::elect_one()) {
 #pragma unroll
-                        for (int ks = 0; ks < D / 16; ++ks) {
-                            constexpr uint32_t kCb = kTcColBlockBytes;
-                            const uint32_t off = ((ks >> 2) * kCb + (ks & 3) * 32) >> 4;
-                            tc::mma_bf16_tmem_a(tS, tQ + 8u * ks, kd + off, kIdS, ks > 0);
+                            for (int ks = 0; ks < D / 16; ++ks) {
+                                constexpr uint32_t kCb = kTcColBlockBytes;
+                                const uint32_t off = ((ks >> 2) * kCb + (ks & 3) * 32) >> 4;
+                                tc::mma_bf16_tmem_a(tS, tQ + 8u * ks, kd + off, kIdS, ks > 0);
+                            }
+                            tc::commit(bar(kBarSFull + (b & 1)));
                         }
-                        tc::commit(bar(kBarSFull + (b & 1)));
                         if (++st == kMmaStages) {
                             st = 0;
                             ph ^= 1;
@@ -1611,32 +1613,31 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                     // PV of the item's blocks into O (buffer k & 1)
                     const uint32_t tO = tmem + kTmemO + 128u * (k & 1);
                     for (int i = 0; i < nb; ++i, ++b) {
-                        if (!wait(kBarPFull + (b & 1), b >> 1) ||
-                            // the O buffer was last used by item k - 2: its epilogue must be done
-                            (i == 0 && k >= 2 && !wait(kBarOEmpty + (k & 1), (k >> 1) - 1))) {
-                            ok = false;
-                            break;
-                        }
+                        if (failed()) break;
+                        wait(kBarPFull + (b & 1), b >> 1);
+                        // the O buffer was last used by item k - 2: its epilogue must be done
+                        if (i == 0 && k >= 2) wait(kBarOEmpty + (k & 1), (k >> 1) - 1);
                         tc::fence_after_sync();
                         const uint32_t tP = tmem + kTmemS + 64u * (b & 1);
                         const uint64_t vd = desc_v + static_cast<uint64_t>(st * kStageStep);
+                        if (tc::elect_one()) {
 #pragma unroll
-                        for (int kk = 0; kk < kTcBlockTokens / 16; ++kk)
-                            tc::mma_bf16_tmem_a(tO, tP + 8u * kk,
-                                                vd + static_cast<uint32_t>((kk * 2048) >> 4), kIdPV,
-                                                i > 0 || kk > 0);
-                        // S(b) completed before P(b) was written: both products
-                        // of the stage are done when these arrive
-                        tc::commit(bar((kF8 ? kBarCvEmpty : kBarKvEmpty) + st));
-                        tc::commit(bar(kBarPvDone + (b & 1)));
-                        if (i == nb - 1) tc::commit(bar(kBarOFull + (k & 1)));
+                            for (int kk = 0; kk < kTcBlockTokens / 16; ++kk)
+                                tc::mma_bf16_tmem_a(tO, tP + 8u * kk,
+                                                    vd + static_cast<uint32_t>((kk * 2048) >> 4), kIdPV,
+                                                    i > 0 || kk > 0);
+                            // S(b) completed before P(b) was written: both
+                            // products of the stage are done when these arrive
+                            tc::commit(bar((kF8 ? kBarCvEmpty : kBarKvEmpty) + st));
+                            tc::commit(bar(kBarPvDone + (b & 1)));
+                            if (i == nb - 1) tc::commit(bar(kBarOFull + (k & 1)));
+                        }
                         if (++st == kMmaStages) st = 0;
                     }
                 }
             }
-            if (!ok) tc_fail(a, abort_flag, kSiteConsumerFull);
             // every MMA of both issuers must finish before TMEM is freed
-            tc::commit(bar(kBarDrain));
+            if (tc::elect_one()) tc::commit(bar(kBarDrain));
             dev::mbar_wait_bounded(bar(kBarDrain), 0, kDrainLimitNs, nullptr);
         }
         __syncwarp();
@@ -1971,9 +1972,9 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
 //   warp 10     scheduler: pulls pairs and stages their metadata
 //   warp 8      producer: TMA of each block of the pair's pages, once, into
 //               a 4-stage ring
-//   warp 9      S issuer (one thread): S_t = Q_t K^T for t = A, B of a block,
+//   warp 9      S issuer (one lane): S_t = Q_t K^T for t = A, B of a block,
 //               A and B from shared memory
-//   warp 11     PV issuer (one thread): O_t += P_t V; the stage goes back to
+//   warp 11     PV issuer (one lane): O_t += P_t V; the stage goes back to
 //               the producer after the block's last PV
 //   warps 0-3   tile A: softmax (thread r owns row r, TMEM lane r), the next
 //               pair's Q rows into shared memory, then the row's (m, l) and O
@@ -2156,57 +2157,61 @@ __device__ void prefix_cta_tc_pair(const KvMaps *maps, const AttnArgs &a, uint8_
                                            kDrainLimitNs, nullptr);
     } else if (warp == kTcMmaWarp || warp == kTcPvWarp) {
         // ------------------------------------------------------------ MMA issuers
-        if (lane == 0) {
+        {
+            // (each warp runs the loop, one elected lane issues: see elect_one)
             constexpr uint32_t kIdS = tc::idesc_bf16_f32(kTcRows, kTcBlockTokens, false);
             constexpr uint32_t kIdPV = tc::idesc_bf16_f32(kTcRows, D, true);
+            // A wait that runs out leaves its mark, and the warp goes on together
+            // to the next point where it looks (lanes that part would leave the
+            // others waiting in elect.sync; what is issued in between works on
+            // this CTA's own memory and is thrown away).
+            bool bad = false;
             auto wait = [&](int i, int parity) {
-                return tc_wait(bar(i), static_cast<uint32_t>(parity & 1), limit, abort_flag);
+                if (!tc_wait(bar(i), static_cast<uint32_t>(parity & 1), limit, abort_flag)) {
+                    tc_fail(a, abort_flag, kSiteConsumerFull);
+                    bad = true;
+                }
             };
+            auto failed = [&]() { return __any_sync(0xffffffffu, bad) != 0; };
             const uint64_t desc_k = tc::smem_desc_sw128(ring, 16, 1024);
             const uint64_t desc_v = tc::smem_desc_sw128(ring + kTcKBytes, kTcColBlockBytes, 1024);
-            const uint64_t desc_q[2] = {tc::smem_desc_sw128(ring + kTpQOffset, 16, 1024),
-                                        tc::smem_desc_sw128(ring + kTpQOffset + kTpQBytes, 16, 1024)};
+            const uint64_t desc_q = tc::smem_desc_sw128(ring + kTpQOffset, 16, 1024);
             constexpr uint32_t kStageStep = kTcStageBytes >> 4;
-            bool ok = true;
             int st = 0, ph = 0;              // stage of the block and the stage's phase parity
             int u[2] = {0, 0};               // blocks of each tile so far
             int j[2] = {0, 0};               // pairs in which each tile had rows
-            for (int k = 0; ok; ++k) {
+            for (int k = 0;; ++k) {
                 const int ms = k % kTcMeta;
-                if (!wait(kPbMetaFull + ms, k / kTcMeta)) {
-                    ok = false;
-                    break;
-                }
-                if (meta[ms].id < 0) break;
+                wait(kPbMetaFull + ms, k / kTcMeta);
+                if (failed() || meta[ms].id < 0) break;
                 const bool on[2] = {true, meta[ms].itB.nrows > 0};
                 const int nb = tc_blocks(meta[ms].it.num_pages);
                 if (warp == kTcMmaWarp) {
-                    for (int t = 0; t < 2 && ok; ++t)
-                        if (on[t] && !wait(kPbQReady + t, j[t])) ok = false;
-                    if (ok) tc::fence_after_sync();
-                    for (int i = 0; i < nb && ok; ++i) {
-                        if (!wait(kPbKvFull + st, ph)) {
-                            ok = false;
-                            break;
-                        }
+                    for (int t = 0; t < 2; ++t)
+                        if (on[t]) wait(kPbQReady + t, j[t]);
+                    tc::fence_after_sync();
+                    for (int i = 0; i < nb; ++i) {
+                        if (failed()) break;
+                        wait(kPbKvFull + st, ph);
                         const uint64_t kd = desc_k + static_cast<uint64_t>(st * kStageStep);
+#pragma unroll
                         for (int t = 0; t < 2; ++t) {
                             if (!on[t]) continue;
                             const int buf = u[t] & 1;
                             // the buffer holds the tile's P of two blocks back until its PV is done
-                            if (u[t] >= 2 && !wait(kPbPvDone + 2 * t + buf, (u[t] - 2) >> 1)) {
-                                ok = false;
-                                break;
-                            }
+                            if (u[t] >= 2) wait(kPbPvDone + 2 * t + buf, (u[t] - 2) >> 1);
                             tc::fence_after_sync();
                             const uint32_t tS = tmem + kTmemS + 128u * t + 64u * buf;
+                            const uint64_t qd = desc_q + static_cast<uint64_t>(t * (kTpQBytes >> 4));
+                            if (tc::elect_one()) {
 #pragma unroll
-                            for (int ks = 0; ks < D / 16; ++ks) {
-                                const uint32_t koff = ((ks >> 2) * kTcColBlockBytes + (ks & 3) * 32) >> 4;
-                                const uint32_t qoff = ((ks >> 2) * kTpQColBlockBytes + (ks & 3) * 32) >> 4;
-                                tc::mma_bf16(tS, desc_q[t] + qoff, kd + koff, kIdS, ks > 0);
+                                for (int ks = 0; ks < D / 16; ++ks) {
+                                    const uint32_t koff = ((ks >> 2) * kTcColBlockBytes + (ks & 3) * 32) >> 4;
+                                    const uint32_t qoff = ((ks >> 2) * kTpQColBlockBytes + (ks & 3) * 32) >> 4;
+                                    tc::mma_bf16(tS, qd + qoff, kd + koff, kIdS, ks > 0);
+                                }
+                                tc::commit(bar(kPbSFull + 2 * t + buf));
                             }
-                            tc::commit(bar(kPbSFull + 2 * t + buf));
                             ++u[t];
                         }
                         if (++st == kTpStages) {
@@ -2215,42 +2220,41 @@ __device__ void prefix_cta_tc_pair(const KvMaps *maps, const AttnArgs &a, uint8_
                         }
                     }
                 } else {
-                    for (int i = 0; i < nb && ok; ++i) {
+                    for (int i = 0; i < nb; ++i) {
+                        if (failed()) break;
                         const uint64_t vd = desc_v + static_cast<uint64_t>(st * kStageStep);
+#pragma unroll
                         for (int t = 0; t < 2; ++t) {
                             if (!on[t]) continue;
                             const int buf = u[t] & 1;
-                            if (!wait(kPbPFull + 2 * t + buf, u[t] >> 1) ||
-                                // the tile's O was last used by its previous pair: stored?
-                                (i == 0 && j[t] > 0 && !wait(kPbOEmpty + t, j[t] - 1))) {
-                                ok = false;
-                                break;
-                            }
+                            wait(kPbPFull + 2 * t + buf, u[t] >> 1);
+                            // the tile's O was last used by its previous pair: stored?
+                            if (i == 0 && j[t] > 0) wait(kPbOEmpty + t, j[t] - 1);
                             tc::fence_after_sync();
                             const uint32_t tO = tmem + kTmemO + 128u * t;
                             const uint32_t tP = tmem + kTmemS + 128u * t + 64u * buf;
+                            if (tc::elect_one()) {
 #pragma unroll
-                            for (int kk = 0; kk < kTcBlockTokens / 16; ++kk)
-                                tc::mma_bf16_tmem_a(tO, tP + 8u * kk,
-                                                    vd + static_cast<uint32_t>((kk * 2048) >> 4), kIdPV,
-                                                    i > 0 || kk > 0);
-                            tc::commit(bar(kPbPvDone + 2 * t + buf));
-                            if (i == nb - 1) tc::commit(bar(kPbOFull + t));
+                                for (int kk = 0; kk < kTcBlockTokens / 16; ++kk)
+                                    tc::mma_bf16_tmem_a(tO, tP + 8u * kk,
+                                                        vd + static_cast<uint32_t>((kk * 2048) >> 4), kIdPV,
+                                                        i > 0 || kk > 0);
+                                tc::commit(bar(kPbPvDone + 2 * t + buf));
+                                if (i == nb - 1) tc::commit(bar(kPbOFull + t));
+                            }
                             ++u[t];
                         }
-                        if (!ok) break;
                         // both tiles' products of the stage are done when this arrives
                         // (each S completed before its P was written)
-                        tc::commit(bar(kPbKvEmpty + st));
+                        if (tc::elect_one()) tc::commit(bar(kPbKvEmpty + st));
                         if (++st == kTpStages) st = 0;
                     }
                 }
                 for (int t = 0; t < 2; ++t)
                     if (on[t]) ++j[t];
             }
-            if (!ok) tc_fail(a, abort_flag, kSiteConsumerFull);
             // every MMA of both issuers must finish before TMEM is freed
-            tc::commit(bar(kPbDrain));
+            if (tc::elect_one()) tc::commit(bar(kPbDrain));
             dev::mbar_wait_bounded(bar(kPbDrain), 0, kDrainLimitNs, nullptr);
         }
         __syncwarp();
