@@ -59,6 +59,7 @@
 
 #include "device_common.cuh"
 #include "tcgen05.cuh"
+#include "tile_common.cuh"
 
 namespace parason {
 namespace {
@@ -169,8 +170,8 @@ __device__ __forceinline__ void load_suffix_page(uint32_t dst, const KvMaps &map
     const uint64_t pol = dev::l2_evict_first_policy();
     if constexpr (S::kSeg > 1) {
         const int ph = row / kPageSize;
-        dev::tma_load_4d_hint(dst, &maps.k_page, 0, 0, 0, ph, bar, pol);
-        dev::tma_load_4d_hint(dst + S::kPageBytes, &maps.v_page, 0, 0, 0, ph, bar, pol);
+        dev::tma_load_4d_hint(dst, &maps.k_box, 0, 0, 0, ph, bar, pol);
+        dev::tma_load_4d_hint(dst + S::kPageBytes, &maps.v_box, 0, 0, 0, ph, bar, pol);
     } else {
         dev::tma_load_3d_hint(dst, &maps.k, 0, 0, row, bar, pol);
         dev::tma_load_3d_hint(dst + S::kPageBytes, &maps.v, 0, 0, row, bar, pol);
@@ -200,58 +201,6 @@ __device__ __forceinline__ int out_col(int nt, int e, int tig) {
         return nt * 8 + 2 * tig + (e & 1);
     else
         return 16 * (2 * tig + (e & 1)) + nt;
-}
-
-__device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint32_t two_bytes) {
-    uint32_t out;
-    asm("{\n\t.reg .b16 lo, hi;\n\t"
-        "mov.b32 {lo, hi}, %1;\n\t"
-        "cvt.rn.f16x2.e4m3x2 %0, lo;\n\t}"
-        : "=r"(out)
-        : "r"(two_bytes));
-    return out;
-}
-
-// Four e4m3 values (one word) widened exactly to two f16 pairs: bytes 0-1
-// to `lo`, bytes 2-3 to `hi`.
-__device__ __forceinline__ void e4m3x4_to_f16x2x2(uint32_t four_bytes, uint32_t &lo, uint32_t &hi) {
-    asm("{\n\t.reg .b16 l, h;\n\t"
-        "mov.b32 {l, h}, %2;\n\t"
-        "cvt.rn.f16x2.e4m3x2 %0, l;\n\t"
-        "cvt.rn.f16x2.e4m3x2 %1, h;\n\t}"
-        : "=r"(lo), "=r"(hi)
-        : "r"(four_bytes));
-}
-
-// A bf16 pair of q narrowed to an f16 pair for the e4m3 MMAs.  The f16
-// values are exact for |q| < 65504 (tiny values lose low bits); an element
-// of magnitude 65520 or more (including inf) would round to inf, so `big` is
-// set and the caller reports PARASON_ERANGE rather than returning a silently
-// wrong result.  NaN is passed through and not flagged.
-__device__ __forceinline__ uint32_t q_pair_to_f16(uint32_t two, bool &big) {
-    const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162 *>(&two);
-    const float lo = __low2float(b), hi = __high2float(b);
-    big |= fmaxf(fabsf(lo), fabsf(hi)) >= 65520.f;
-    return dev::pack_f16(lo, hi);
-}
-
-// Record PARASON_ERANGE once per warp if any lane saw an out-of-range q.
-__device__ __forceinline__ void report_q_range(const AttnArgs &a, bool big, int lane) {
-    if (__any_sync(0xffffffffu, big) && lane == 0) dev::record_error(a.err, PARASON_ERANGE, kSiteQRange);
-}
-
-__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
-    uint32_t v;
-    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr));
-    return v;
-}
-
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "r"(addr));
-    return v;
 }
 
 // Online softmax over one page's scores s (two n-tiles of 8 tokens), then
@@ -1240,61 +1189,16 @@ static_assert(kMaxSuffixWarps <= kThreads / 32, "every suffix-pass warp exists")
 struct TcMeta {
     WorkItem it;
     int32_t id;                      // -1: the queue is empty
-    int32_t key0;                    // causal item: its first key's token index, else -1
-    int32_t key0B;                   // pair mode: the same for the second tile
-    int32_t pad;
+    int32_t pad[3];
     WorkItem itB;                    // pair mode: the second tile (no rows: none)
     int32_t rows[kTcMetaPages];      // TMA row of each page
     int32_t leaves[kTcRows];         // branch of rows [g i, g i + g)
     int32_t leavesB[kTcRows];        // pair mode: the same for the second tile
-    // leading valid tokens of each 64-token block (64 but where a node ends
-    // inside the item: a prefill piece over a path pads each node that ends
-    // inside a page with zero-filled pages up to the next block); the item's
-    // last block also goes by last_valid
-    uint8_t block_valid[kTcMetaPages / 4];
 };
 
-// causal mask: -1 when the item's rows see all of its keys
-constexpr int32_t kNoKey0 = -1;
-
-// 32 consecutive fp32 values of one partial row (128 bytes, 32-byte
-// aligned), scaled, as four 32-byte stores: every store fills whole sectors
-// (16-byte stores from the 32 rows of a warp left each sector to be filled
-// by two instructions).
-__device__ __forceinline__ void store_row32(float *dst, const uint32_t (&v)[32], float scale) {
-#pragma unroll
-    for (int q = 0; q < 32; q += 8)
-        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + q),
-                     "f"(__uint_as_float(v[q]) * scale), "f"(__uint_as_float(v[q + 1]) * scale),
-                     "f"(__uint_as_float(v[q + 2]) * scale), "f"(__uint_as_float(v[q + 3]) * scale),
-                     "f"(__uint_as_float(v[q + 4]) * scale), "f"(__uint_as_float(v[q + 5]) * scale),
-                     "f"(__uint_as_float(v[q + 6]) * scale), "f"(__uint_as_float(v[q + 7]) * scale)
-                     : "memory");
-}
-
-// An item's page rows into its metadata slot: the TMA row of every page
-// (padding pages carry the first row past the pool, which TMA fills with
-// zeros), and the leading valid tokens of every block, from the low 4 bits
-// of the stream rows (16 - the valid tokens of a page that ends a node;
-// a TMA row (page * H_kv + kv head) * 16 leaves them zero).
-__device__ __forceinline__ void stage_item_rows(TcMeta &m, const int32_t *src, int np, int kv_rows,
-                                                int lane) {
-    // lane b takes block b: its 4 rows are loaded before any is looked at
-    for (int b = lane; b * 4 < np; b += 32) {
-        int32_t row[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) row[j] = b * 4 + j < np ? src[b * 4 + j] : kv_rows;
-        int v = 0;
-        bool open = true;                                  // no node has ended in the block yet
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int low = row[j] & (kPageSize - 1);
-            if (open && row[j] < kv_rows) v += kPageSize - low;
-            open = open && row[j] < kv_rows && low == 0;   // padding, or a node's last page
-            if (b * 4 + j < np) m.rows[b * 4 + j] = row[j] & ~(kPageSize - 1);
-        }
-        m.block_valid[b] = static_cast<uint8_t>(v);
-    }
+// An item's page rows (TMA rows) into its metadata slot.
+__device__ __forceinline__ void stage_item_rows(TcMeta &m, const int32_t *src, int np, int lane) {
+    for (int i = lane; i < np; i += 32) m.rows[i] = src[i];
 }
 
 // barrier slots (8 bytes each) in the CTA's barrier area
@@ -1375,26 +1279,6 @@ __device__ __forceinline__ void convert_block_e4m3(uint32_t src, uint32_t dst, i
     }
 }
 
-__device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity, long long limit,
-                                        volatile int *abort) {
-    return dev::mbar_wait_bounded(bar, parity, limit, abort);
-}
-
-// one warp: lane 0 waits, the warp agrees on the outcome
-__device__ __forceinline__ bool tc_warp_wait(uint32_t bar, uint32_t parity, long long limit,
-                                             volatile int *abort, int lane) {
-    int ok = 1;
-    if (lane == 0) ok = tc_wait(bar, parity, limit, abort) ? 1 : 0;
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
-}
-
-__device__ __forceinline__ void tc_fail(const AttnArgs &a, volatile int *abort, int site) {
-    if (!*abort) {
-        *abort = 1;
-        dev::record_error(a.err, PARASON_ETIMEOUT, site);
-    }
-}
-
 __device__ __forceinline__ int tc_blocks(int num_pages) {
     return (num_pages + kTcBlockPages - 1) / kTcBlockPages;
 }
@@ -1433,11 +1317,8 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                     }
                     id = -1;
                 } else {
-                    if (lane == 0) {
-                        m.it = it;
-                        m.key0 = a.item_key0 ? a.item_key0[id] : kNoKey0;
-                    }
-                    stage_item_rows(m, a.stream_rows + a.item_rows[id], it.num_pages, a.kv_rows, lane);
+                    if (lane == 0) m.it = it;
+                    stage_item_rows(m, a.stream_rows + a.item_rows[id], it.num_pages, lane);
                     const int nbr = (it.nrows + a.group - 1) / a.group;
                     const int32_t *lv = a.dfs_leaf + it.leaf_lo + it.row0 / a.group;
                     for (int i = lane; i < nbr; i += 32) m.leaves[i] = lv[i];
@@ -1657,18 +1538,13 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
             const int nb = tc_blocks(it.num_pages);
             const int tokens = (it.num_pages - 1) * kPageSize + it.last_valid;
             const uint32_t tO = lane_base + kTmemO + 128u * (k & 1);
-            // causal item (tree-masked prefill): the row's token, relative to
-            // the item's first key, is the last key it sees
-            const int key0 = meta[ms].key0;
-            const int t_rel = key0 == kNoKey0 ? (1 << 30) : (it.row0 + r) / a.group - key0;
             // e4m3 K: the kv head's scale goes into the logits
             const float sl = kF8 ? a.scale_log2 * a.k_scale[it.kv_head] : a.scale_log2;
             float m_use = -INFINITY, l = 0.f;
             bool ok = true;
             for (int i = 0; i < nb; ++i) {
                 const int b = blk + i;
-                const int valid = min(static_cast<int>(meta[ms].block_valid[i]), tokens - i * kTcBlockTokens);
-                const int seen = min(valid, t_rel - i * kTcBlockTokens + 1);   // keys the row sees
+                const int valid = tokens - i * kTcBlockTokens;   // of the block's keys (64 or more: all)
                 const uint32_t tS = lane_base + kTmemS + 64u * (b & 1);
                 if (!tc_warp_wait(bar(kBarSFull + (b & 1)), (b >> 1) & 1, limit, abort_flag, lane)) {
                     ok = false;
@@ -1679,14 +1555,13 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                 tc::ld32(tS, sr[0]);
                 tc::ld32(tS + 32, sr[1]);
                 tc::wait_ld();
-                // raw scores; keys the row does not see (past the item's last
-                // token, or past the row's own token in a causal item) -inf
+                // raw scores; keys past the item's last token -inf
                 float x[64];
 #pragma unroll
                 for (int j = 0; j < 64; ++j) x[j] = __uint_as_float(sr[j >> 5][j & 31]);
-                if (seen < kTcBlockTokens) {
+                if (valid < kTcBlockTokens) {
 #pragma unroll
-                    for (int j = 0; j < 64; ++j) x[j] = j < seen ? x[j] : -INFINITY;
+                    for (int j = 0; j < 64; ++j) hide_from(x[j], j, valid);
                 }
                 // the block's max in the log2 domain (sl > 0)
                 float mr = x[0];
@@ -1705,7 +1580,6 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                     }
                     tc::fence_after_sync();
                     const float m_new = fmaxf(m_use, mb);
-                    // (a row with no visible key yet keeps m = -inf and alpha 1)
                     const float alpha = m_new == m_use ? 1.f : dev::fast_exp2(m_use - m_new);
 #pragma unroll
                     for (int c = 0; c < D / 32; ++c) {
@@ -1721,7 +1595,6 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                     m_use = m_new;
                 }
                 // P = 2^(x - m) as bf16 pairs over the first 32 columns of S
-                // (0 for a row that has seen no key: every x is -inf)
                 const float m_ref = m_use == -INFINITY ? 0.f : m_use;
                 // 2^(x sl - m) with pairs of fp32 lanes: one packed FMA per
                 // two exponents, and two running sums
@@ -2070,10 +1943,8 @@ __device__ void prefix_cta_tc_pair(const KvMaps *maps, const AttnArgs &a, uint8_
                     if (lane == 0) {
                         m.it = it;
                         m.itB = itB;
-                        m.key0 = a.item_key0 ? a.item_key0[id] : kNoKey0;
-                        m.key0B = a.item_key0 ? a.item_key0[id + 1] : kNoKey0;
                     }
-                    stage_item_rows(m, a.stream_rows + a.item_rows[id], it.num_pages, a.kv_rows, lane);
+                    stage_item_rows(m, a.stream_rows + a.item_rows[id], it.num_pages, lane);
                     const int nbr = (it.nrows + a.group - 1) / a.group;
                     const int32_t *lv = a.dfs_leaf + it.leaf_lo + it.row0 / a.group;
                     for (int i = lane; i < nbr; i += 32) m.leaves[i] = lv[i];
@@ -2320,14 +2191,11 @@ __device__ void prefix_cta_tc_pair(const KvMaps *maps, const AttnArgs &a, uint8_
                 const WorkItem it = tile_of(m);
                 const int nb = tc_blocks(it.num_pages);
                 const int tokens = (it.num_pages - 1) * kPageSize + it.last_valid;
-                const int key0 = t == 0 ? m.key0 : m.key0B;
-                const int t_rel = key0 == kNoKey0 ? (1 << 30) : (it.row0 + r) / a.group - key0;
                 float m_use = -INFINITY, l = 0.f;
                 for (int i = 0; i < nb; ++i) {
                     const int buf = u & 1;
                     const uint32_t tS = lane_base + kTmemS + 128u * t + 64u * buf;
-                    const int valid = min(static_cast<int>(m.block_valid[i]), tokens - i * kTcBlockTokens);
-                    const int seen = min(valid, t_rel - i * kTcBlockTokens + 1);
+                    const int valid = tokens - i * kTcBlockTokens;
                     if (!tc_warp_wait(bar(kPbSFull + 2 * t + buf), (u >> 1) & 1, limit, abort_flag, lane)) {
                         ok = false;
                         break;
@@ -2350,9 +2218,9 @@ __device__ void prefix_cta_tc_pair(const KvMaps *maps, const AttnArgs &a, uint8_
                     float x[64];
 #pragma unroll
                     for (int q = 0; q < 64; ++q) x[q] = __uint_as_float(sr[q >> 5][q & 31]);
-                    if (seen < kTcBlockTokens) {
+                    if (valid < kTcBlockTokens) {
 #pragma unroll
-                        for (int q = 0; q < 64; ++q) x[q] = q < seen ? x[q] : -INFINITY;
+                        for (int q = 0; q < 64; ++q) hide_from(x[q], q, valid);
                     }
                     float mr = x[0];
 #pragma unroll
@@ -2511,8 +2379,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         dev::prefetch_tensormap(&maps.k);
         dev::prefetch_tensormap(&maps.v);
         if constexpr (S::kSeg > 1) {
-            dev::prefetch_tensormap(&maps.k_page);
-            dev::prefetch_tensormap(&maps.v_page);
+            dev::prefetch_tensormap(&maps.k_box);
+            dev::prefetch_tensormap(&maps.v_box);
         }
     }
     if constexpr (kTcPrefix) {

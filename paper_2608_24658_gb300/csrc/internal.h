@@ -95,6 +95,11 @@ struct AttnArgs {
     // one piece (position k: items 2k and 2k + 1, the second without rows
     // when the piece has one tile), run by the tcgen05 tile in pair mode
     int32_t tc_pairs;
+    // a prefill whose pairs each hold their rows' whole paths (plan.cpp:
+    // direct): the attention kernel writes out and lse (null: none) itself and
+    // no merge runs; out is null otherwise
+    void *out;
+    float *lse;
 };
 
 struct MergeArgs {
@@ -122,12 +127,14 @@ cudaError_t attn_mma_ctas_per_sm(int head_dim, int mode, int *ctas_per_sm);
 // TMA views of the K and V pools.  k / v: one box is one 128-byte column
 // block of one page of one kv head (16 rows).  k_run / v_run: one box is the
 // same column block of kTcRunPages consecutive pages of one kv head, for
-// blocks whose pages are consecutive in the pool.  k_page / v_page: one box
-// is a whole page of one kv head, its column blocks one after another (the
-// layout the per-block boxes of k / v give).
+// blocks whose pages are consecutive in the pool.  k_box / v_box: one box is
+// kBoxPages pages of one kv head that are consecutive in the pool, its column
+// blocks one after another (the layout the per-block boxes of k / v give):
+// one page in a decode plan, a 128-token block in a prefill plan.
 constexpr int kTcRunPages = 4;
+constexpr int kDecodeBoxPages = 1, kPrefillBoxPages = 8;
 struct KvMaps {
-    CUtensorMap k, v, k_run, v_run, k_page, v_page;
+    CUtensorMap k, v, k_run, v_run, k_box, v_box;
 };
 
 // Kernel launchers; each returns the launch's cudaError_t.
@@ -135,6 +142,8 @@ cudaError_t launch_attn_bf16(const AttnArgs &a, const KvMaps &maps, int head_dim
                              cudaStream_t stream);
 cudaError_t launch_attn_fp8(const AttnArgs &a, const KvMaps &maps, int head_dim,
                             cudaStream_t stream);
+// tree-masked prefill (bf16 or e4m3 KV at head_dim 128)
+cudaError_t launch_prefill(const AttnArgs &a, const KvMaps &maps, int mode, cudaStream_t stream);
 cudaError_t launch_attn_fp32(const AttnArgs &a, const float *k_pages, const float *v_pages,
                              int head_dim, cudaStream_t stream);
 cudaError_t launch_merge(const MergeArgs &a, int head_dim, int mode, bool programmatic,

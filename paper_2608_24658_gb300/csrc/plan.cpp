@@ -54,17 +54,21 @@ constexpr int kWideBlockPages = 4;      // prefix pieces are whole 64-token bloc
 // 39.8 -> 39.2 us, long prefix 854.5 -> 843 us (e4m3 KV 655.4 -> 600.2
 // us), batched 2460 -> 2447 us.
 constexpr int64_t kWidePiecesPerCta = 1;
-// A prefill's queue is the whole launch, and nothing evens out the prefix
-// CTAs' ends: its piece length is the one, of a few candidates, under which
-// the queue, simulated, empties first.  An entry's start and its O cost
-// about kPieceStartPages pages (join prefill, 8 -> 16 pieces per path: the
-// kernel went from 606 to 672 us for 1024 more pairs on 152 CTAs, about 38
-// pages of a pair each); a lone tile of a pair kLoneTileShare of a pair's
-// time.
-constexpr double kPieceStartPages = 32.0;
-constexpr double kLoneTileShare = 0.6;
-constexpr int kPieceCountCandidates = 16;
-constexpr int64_t kPieceLengthSteps = 16;   // lengths tried per piece count, 4 pages apart
+// A prefill's queue is the whole launch, and nothing evens out its CTAs' ends:
+// its piece length is the one, of a few candidates, under which the queue,
+// simulated, empties first (prefill_cut).  In pages of a pair (0.21 us with
+// bf16 KV): an entry's start and its O cost a CTA kPieceStartPages (43-block
+// pieces took 82 us where 281-block ones took 1.67 us a block); its partial
+// rows, written and read back by the merge, every CTA another
+// kPiecePartialPages / num_sms; the merge itself kMergePages, unless every
+// entry holds its rows' whole paths; a pair without a second tile takes
+// kLoneTileShare of a pair's time.
+constexpr double kPieceStartPages = 28.0;
+constexpr double kPiecePartialPages = 39.0;
+constexpr double kMergePages = 28.0;
+constexpr double kLoneTileShare = 0.85;
+constexpr int kPieceCounts = 8;
+constexpr int kPrefillBlockPages = parason::kPrefillBoxPages;   // a prefill tile's blocks
 // suffix pieces: about this many per warp of the launch (at least
 // kMinPiecePages and at most kMaxPiecePages pages).  Same-box A/B against
 // 3: two-level step 79.7 -> 78.8 us, the Llama-3 shape level (its pieces
@@ -124,28 +128,35 @@ void piece_split(int64_t pages, int64_t chunk, int64_t align, int64_t &per, int6
     n = (pages + per - 1) / per;
 }
 
-// Time, in pages, for `ctas` CTAs to empty a prefix queue whose (pages,
-// tiles) groups are cut into pieces of at most `chunk` pages.  The queue
-// hands its entries out longest first, the first `ctas` to the CTAs that own
-// them, each later one to the CTA that frees first.  An entry is a tile, or
-// with pairs two tiles (a lone tile at kLoneTileShare of a pair's time), and
-// costs its pages plus kPieceStartPages for its start and its O.
-double prefix_queue_time(const std::vector<std::pair<int64_t, int32_t>> &groups, int64_t chunk,
-                         int32_t ctas, bool pairs) {
+// A prefill's runs of one (chunk, kv head, page list): its pages, tiles and rows.
+struct PrefillGroup {
+    int64_t pages;
+    int32_t tiles, rows;
+};
+
+// Time, in pages, for `ctas` CTAs to empty a prefill queue whose groups are
+// cut into pieces of `chunk` pages, and the partial rows that takes.  The
+// queue hands its pairs out longest first, the first `ctas` to the CTAs that
+// own them, each later one to the CTA that frees first.  A run is cut into
+// whole pieces and a remainder: equal pieces would give the CTAs that take n
+// + 1 of them a whole piece more than those that take n, where long pieces
+// and remainders even out with the fewest pieces.
+double prefill_queue_time(const std::vector<PrefillGroup> &groups, int64_t chunk, int32_t ctas,
+                          bool whole_paths, int64_t &rows) {
     std::vector<std::pair<int64_t, double>> entries;   // (pages, time)
-    for (const auto &g : groups) {
-        int64_t per = 0, n = 0;
-        piece_split(g.first, chunk, kWideBlockPages, per, n);
-        const int32_t full = pairs ? g.second / 2 : g.second;
-        const int32_t lone = pairs ? g.second % 2 : 0;
-        for (int64_t k = 0; k < n; ++k) {
-            const int64_t np = std::min(per, g.first - k * per);
-            for (int32_t t = 0; t < full; ++t)
-                entries.emplace_back(np, static_cast<double>(np) + kPieceStartPages);
-            for (int32_t t = 0; t < lone; ++t)
-                entries.emplace_back(np, kLoneTileShare * static_cast<double>(np) + kPieceStartPages);
+    rows = 0;
+    bool whole = true;                                 // no group is cut
+    for (const PrefillGroup &g : groups)
+        for (int64_t left = g.pages; left > 0;) {
+            whole = whole && left <= chunk;
+            const int64_t np = std::min(left, chunk);
+            left -= np;
+            rows += g.rows;
+            const double t = static_cast<double>((np + kPrefillBlockPages - 1) / kPrefillBlockPages *
+                                                 kPrefillBlockPages);
+            for (int32_t k = 0; k < g.tiles / 2; ++k) entries.emplace_back(np, t + kPieceStartPages);
+            if (g.tiles % 2) entries.emplace_back(np, kLoneTileShare * t + kPieceStartPages);
         }
-    }
     std::stable_sort(entries.begin(), entries.end(),
                      [](const auto &a, const auto &b) { return a.first > b.first; });
     std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
@@ -160,7 +171,47 @@ double prefix_queue_time(const std::vector<std::pair<int64_t, int32_t>> &groups,
         free_at.push(t1);
         end = std::max(end, t1);
     }
-    return end;
+    if (whole && whole_paths && entries.size() <= static_cast<size_t>(ctas)) return end;
+    return end + kMergePages + kPiecePartialPages * static_cast<double>(entries.size()) / ctas;
+}
+
+// The piece length of a prefill plan.  Candidates: the longest run cut into n
+// equal pieces, and one CTA's share of the work cut into n, or a little
+// under (a long piece a CTA and the remainders on the CTAs left over).  A cut
+// whose partial rows pass what a decode without a caller's workspace holds is
+// taken only if none stays under it.
+int64_t prefill_cut(const std::vector<PrefillGroup> &groups, int32_t ctas, bool whole_paths,
+                    int64_t max_rows) {
+    int64_t longest = 0, total = 0;
+    for (const PrefillGroup &g : groups) {
+        longest = std::max(longest, g.pages);
+        total += g.pages * ((g.tiles + 1) / 2);
+    }
+    const int64_t share = (total + ctas - 1) / ctas;
+    std::vector<int64_t> cands;
+    for (int64_t n = 1; n <= kPieceCounts; ++n) {
+        cands.push_back((longest + n - 1) / n);
+        for (int64_t pct = 80; pct <= 104; pct += 4) cands.push_back(share * pct / (100 * n));
+    }
+    for (int64_t &c : cands)
+        c = std::min(longest + kPrefillBlockPages - 1, std::max<int64_t>(c, 1) + kPrefillBlockPages - 1) /
+            kPrefillBlockPages * kPrefillBlockPages;
+    std::sort(cands.begin(), cands.end(), std::greater<int64_t>());
+    cands.erase(std::unique(cands.begin(), cands.end()), cands.end());
+    int64_t best = cands.front();
+    double best_t = -1.0;
+    bool best_fits = false;
+    for (int64_t c : cands) {
+        int64_t rows = 0;
+        const double t = prefill_queue_time(groups, c, ctas, whole_paths, rows);
+        const bool fits = rows <= max_rows;
+        if (best_t < 0.0 || (fits && !best_fits) || (fits == best_fits && t < best_t)) {
+            best = c;
+            best_t = t;
+            best_fits = fits;
+        }
+    }
+    return best;
 }
 
 // Rows of one tile: a multiple of g (so a branch's rows never straddle two
@@ -215,6 +266,8 @@ struct parason_plan_s {
     int64_t unique_tokens = 0;
     int64_t path_tokens = 0;
     bool prefill = false;              // a tree-masked prefill plan
+    bool direct = false;               // every pair holds its rows' whole paths and has a CTA of
+                                       // its own: the attention kernel writes the result
     std::vector<int32_t> shard_branch; // sharded plans: global index of each branch
     std::vector<int32_t> item_key0;    // prefill: first key of a causal item, else -1
 
@@ -427,8 +480,8 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
     double wide_cost = 0.0;
     if (prefill) {
         // chunk c: rows (token t, q head r) = t * g + r of every kv head, in
-        // tiles; each tile reads every ancestor in full and its own node up
-        // to the tile's last token
+        // tiles that run in pairs; each pair reads every ancestor in full and
+        // its own node up to the pair's last token
         for (int32_t c = 0; c < num_leaves; ++c) {
             const int32_t n = leaf_node[c];
             const int64_t C = node_len[n];
@@ -492,7 +545,8 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
                     if (node_len[m] == 0) continue;
                     for (int64_t r0 = 0; r0 < R; r0 += rt) {
                         const int64_t nrows = std::min<int64_t>(rt, R - r0);
-                        const int64_t tb = (r0 + nrows) / g;         // tokens [r0 / g, tb)
+                        // the tokens up to the end of the tile's pair
+                        const int64_t tb = std::min<int64_t>(R, (r0 / (2 * rt) + 1) * 2 * rt) / g;
                         Run run;
                         run.node = m;
                         run.head = j;
@@ -559,14 +613,14 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
             ++j;
         return j;
     };
-    // Pairs of tiles: with bf16 KV at head_dim 128, when most prefix
+    // Pairs of tiles: in a prefill always; with bf16 KV at head_dim 128, when most prefix
     // tile-pages sit in pieces of two or more tiles, the tcgen05 tile runs
     // two tiles of a piece against each staged block.  The cost model and
     // the piece length still count tiles one by one (counting a pair as one
     // unit made fewer prefix CTAs and longer pieces, and was slower: long
     // prefix 841.8 -> 853.4 us, 32k prefix tile alone 156.1 -> 232.4 us).
-    p->tc_pairs = false;
-    if (mode == PARASON_BF16 && cfg->head_dim == 128) {
+    p->tc_pairs = prefill;
+    if (!prefill && mode == PARASON_BF16 && cfg->head_dim == 128) {
         int64_t multi = 0, all = 0;
         for (size_t i = 0; i < runs.size();) {
             const size_t j = group_end(i);
@@ -751,34 +805,19 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
                               static_cast<int64_t>(static_cast<double>(narrow_pages) /
                                                    (kNarrowPiecesPerWarp * std::max<int64_t>(1, total_warps)))));
         p->narrow_chunk = narrow_chunk;
-        if (prefill && n_wide > 0) {
-            // candidates: the longest run cut into n pieces, n from the
-            // fewest the tile allows up, and the lengths between that and
-            // the shortest run cut into n pieces (which give the longer runs
-            // n + 1 pieces and the shorter ones n)
-            std::vector<std::pair<int64_t, int32_t>> groups;   // (pages, tiles)
-            int64_t longest = 0, shortest = INT64_MAX;
+        if (prefill && n_wide > 0 && !runs.empty()) {
+            std::vector<PrefillGroup> groups;
             for (size_t i = 0; i < runs.size();) {
                 const size_t j = group_end(i);
-                groups.emplace_back(runs[i].pages, static_cast<int32_t>(j - i));
-                longest = std::max(longest, runs[i].pages);
-                shortest = std::min(shortest, runs[i].pages);
+                int32_t rows = 0;
+                for (size_t t = i; t < j; ++t) rows += runs[t].nrows;
+                groups.push_back({runs[i].pages, static_cast<int32_t>(j - i), rows});
                 i = j;
             }
-            double best = prefix_queue_time(groups, wide_chunk, n_wide, p->tc_pairs);
-            const int64_t n0 = (longest + kMaxTileItemPages - 1) / kMaxTileItemPages;
-            for (int64_t n = n0; n < n0 + kPieceCountCandidates; ++n) {
-                const int64_t hi = (longest + n - 1) / n;
-                const int64_t lo = std::max<int64_t>((shortest + n - 1) / n, hi - kPieceLengthSteps * kWideBlockPages);
-                for (int64_t c0 = hi; c0 >= lo; c0 -= kWideBlockPages) {
-                    const int64_t c = std::min<int64_t>(kMaxTileItemPages, std::max<int64_t>(kWideBlockPages, c0));
-                    const double tq = prefix_queue_time(groups, c, n_wide, p->tc_pairs);
-                    if (tq < best) {
-                        best = tq;
-                        wide_chunk = c;
-                    }
-                }
-            }
+            const int64_t row_bytes = static_cast<int64_t>(cfg->head_dim) * 4 + 8;
+            wide_chunk = prefill_cut(
+                groups, n_wide, mode == PARASON_BF16,   // (e4m3 runs are one node's)
+                (PARASON_NO_ALLOC_SCRATCH_BYTES - 2 * static_cast<int64_t>(kAlign)) / row_bytes);
         }
         // The row tiles of one (node, kv head) read the same pages: their
         // pieces are emitted piece by piece across the tiles, so that the
@@ -790,7 +829,10 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
             const bool pairs = r.wide && p->tc_pairs;
             const int64_t align = r.wide ? kWideBlockPages : 1;
             int64_t per = 0, n = 0;
-            piece_split(r.pages, r.wide ? wide_chunk : narrow_chunk, align, per, n);
+            if (prefill)
+                per = wide_chunk;
+            else
+                piece_split(r.pages, r.wide ? wide_chunk : narrow_chunk, align, per, n);
             for (int64_t pg = 0; pg < r.pages; pg += per) {
                 const int64_t np = std::min(per, r.pages - pg);
                 for (size_t t = i; t < j; ++t) {
@@ -936,6 +978,9 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
         if (p->merge_ent.size() > static_cast<size_t>(INT32_MAX)) return PARASON_EUNSUPPORTED;
         p->merge_rng[k] = make_int2(e0, static_cast<int32_t>(p->merge_ent.size()));
     }
+    p->direct = prefill && !p->items.empty() &&
+                p->wide_queue.size() <= 2 * static_cast<size_t>(p->num_ctas);
+    for (const int2 &rg : p->merge_rng) p->direct = p->direct && rg.y - rg.x == 1;
     for (int32_t b = 0; b < num_leaves && !prefill; ++b)
         for (int32_t n = leaf_node[b]; n >= 0; n = parent[n]) p->path_tokens += node_len[n];
 
@@ -1108,14 +1153,17 @@ parason_status encode_kv_run_map(CUtensorMap *map, const void *pages, int64_t nu
     return r == CUDA_SUCCESS ? PARASON_OK : PARASON_ECUDA;
 }
 
-// The same pool as a 4-D view whose dims are not in stride order: dim0 = 128
+// The same pool as a view whose dims are not in stride order: dim0 = 128
 // bytes of one segment, dim1 = slot in the page (16, stride one token row),
-// dim2 = segment (stride 128 bytes), dim3 = (page * H_kv + kv_head).  One box
-// {seg, 16, nseg, 1} is a whole page of one kv head with its column blocks
-// one after another, each 16 rows of 128 bytes (128-byte swizzle): what nseg
-// boxes of the 3-D view give, in one copy.
-parason_status encode_kv_page_map(CUtensorMap *map, const void *pages, int64_t num_phys,
-                                  int32_t H_kv, int32_t head_dim, int32_t mode) {
+// then for a decode plan dim2 = segment (stride 128 bytes) and dim3 = (page *
+// H_kv + kv_head), and a box {seg, 16, nseg, 1} is a whole page of one kv head
+// with its column blocks one after another, each 16 rows of 128 bytes
+// (128-byte swizzle): what nseg boxes of the 3-D view give, in one copy.  For
+// a prefill plan dim2 = page, dim3 = segment and dim4 = kv head, and a box
+// {seg, 16, kPrefillBoxPages, nseg, 1} is a block of consecutive pages in the
+// same layout, each column block 16 kPrefillBoxPages rows.
+parason_status encode_kv_box_map(CUtensorMap *map, const void *pages, int64_t num_phys,
+                                 int32_t H_kv, int32_t head_dim, int32_t mode, bool prefill) {
     auto fn = encode_fn();
     if (!fn) return PARASON_ECUDA;
     const int esize = (mode == PARASON_FP8_E4M3_KV) ? 1 : 2;
@@ -1123,16 +1171,19 @@ parason_status encode_kv_page_map(CUtensorMap *map, const void *pages, int64_t n
         (mode == PARASON_FP8_E4M3_KV) ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     const int row_bytes = head_dim * esize;
     if (row_bytes % 128 != 0) return PARASON_EUNSUPPORTED;
-    const int nseg = row_bytes / 128;
-    const int seg_elems = 128 / esize;
-    cuuint64_t dims[4] = {static_cast<cuuint64_t>(seg_elems), static_cast<cuuint64_t>(parason::kPageSize),
-                          static_cast<cuuint64_t>(nseg), static_cast<cuuint64_t>(num_phys) * H_kv};
-    cuuint64_t strides[3] = {static_cast<cuuint64_t>(row_bytes), 128,
-                             static_cast<cuuint64_t>(parason::kPageSize) * row_bytes};
-    cuuint32_t box[4] = {static_cast<cuuint32_t>(seg_elems), static_cast<cuuint32_t>(parason::kPageSize),
-                         static_cast<cuuint32_t>(nseg), 1u};
-    cuuint32_t estr[4] = {1, 1, 1, 1};
-    CUresult r = fn(map, dt, 4, const_cast<void *>(pages), dims, strides, box, estr,
+    const cuuint64_t nseg = row_bytes / 128, seg_elems = 128 / esize, slots = parason::kPageSize;
+    const cuuint64_t head_bytes = slots * row_bytes, H = H_kv, P = num_phys;
+    const cuuint64_t dims_d[4] = {seg_elems, slots, nseg, P * H};
+    const cuuint64_t strides_d[3] = {static_cast<cuuint64_t>(row_bytes), 128, head_bytes};
+    const cuuint32_t box_d[4] = {static_cast<cuuint32_t>(seg_elems), parason::kPageSize,
+                                 static_cast<cuuint32_t>(nseg), parason::kDecodeBoxPages};
+    const cuuint64_t dims_p[5] = {seg_elems, slots, P, nseg, H};
+    const cuuint64_t strides_p[4] = {static_cast<cuuint64_t>(row_bytes), head_bytes * H, 128, head_bytes};
+    const cuuint32_t box_p[5] = {static_cast<cuuint32_t>(seg_elems), parason::kPageSize,
+                                 parason::kPrefillBoxPages, static_cast<cuuint32_t>(nseg), 1u};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    CUresult r = fn(map, dt, prefill ? 5 : 4, const_cast<void *>(pages), prefill ? dims_p : dims_d,
+                    prefill ? strides_p : strides_d, prefill ? box_p : box_d, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? PARASON_OK : PARASON_ECUDA;
@@ -1475,6 +1526,10 @@ parason_status parason_attn_decode(parason_plan p, const void *q, const void *k_
         a.item_key0 = p->d_item_key0;
         a.suffix_warps = p->suffix_warps;
         a.tc_pairs = p->tc_pairs ? 1 : 0;
+        if (p->direct) {
+            a.out = out;
+            a.lse = lse;
+        }
         cudaError_t e;
         if (p->cfg.mode == PARASON_FP32) {
             e = parason::launch_attn_fp32(a, static_cast<const float *>(k_pages),
@@ -1490,7 +1545,8 @@ parason_status parason_attn_decode(parason_plan p, const void *q, const void *k_
                     if (st == PARASON_OK)
                         st = encode_kv_run_map(&p->tm.k_run, k_pages, p->num_phys, H, d, mode);
                     if (st == PARASON_OK)
-                        st = encode_kv_page_map(&p->tm.k_page, k_pages, p->num_phys, H, d, mode);
+                        st = encode_kv_box_map(&p->tm.k_box, k_pages, p->num_phys, H, d, mode,
+                                               p->prefill);
                     if (st != PARASON_OK) return st;
                     p->tm_k_ptr = k_pages;
                 }
@@ -1500,14 +1556,16 @@ parason_status parason_attn_decode(parason_plan p, const void *q, const void *k_
                     if (st == PARASON_OK)
                         st = encode_kv_run_map(&p->tm.v_run, v_pages, p->num_phys, H, d, mode);
                     if (st == PARASON_OK)
-                        st = encode_kv_page_map(&p->tm.v_page, v_pages, p->num_phys, H, d, mode);
+                        st = encode_kv_box_map(&p->tm.v_box, v_pages, p->num_phys, H, d, mode,
+                                               p->prefill);
                     if (st != PARASON_OK) return st;
                     p->tm_v_ptr = v_pages;
                 }
                 maps = p->tm;
             }
-            e = (p->cfg.mode == PARASON_BF16) ? parason::launch_attn_bf16(a, maps, d, stream)
-                                              : parason::launch_attn_fp8(a, maps, d, stream);
+            e = p->prefill ? parason::launch_prefill(a, maps, p->cfg.mode, stream)
+                : (p->cfg.mode == PARASON_BF16) ? parason::launch_attn_bf16(a, maps, d, stream)
+                                                : parason::launch_attn_fp8(a, maps, d, stream);
         }
         if (e == cudaErrorNotSupported) return PARASON_EUNSUPPORTED;
         if (e != cudaSuccess) return PARASON_ECUDA;
@@ -1530,7 +1588,9 @@ parason_status parason_attn_decode(parason_plan p, const void *q, const void *k_
     m.queue_start[1] = p->queue_start[1];
     // programmatic dependent launch after the attention kernel: the merge
     // grid is launched while the attention grid drains, and waits for it
-    if (parason::launch_merge(m, d, p->cfg.mode, has_items, stream) != cudaSuccess) return PARASON_ECUDA;
+    if (!p->direct &&
+        parason::launch_merge(m, d, p->cfg.mode, has_items, stream) != cudaSuccess)
+        return PARASON_ECUDA;
     st = record_event(p, 2, stream);
     if (st != PARASON_OK) return st;
     if (p->timing_cap > 0 && p->timing_n < p->timing_cap) p->timing_n++;
@@ -2056,7 +2116,7 @@ parason_status parason_plan_read_timing(parason_plan p, float *attn_ms, float *m
 
 int32_t parason_plan_launches_per_decode(parason_plan p) {
     if (!p || p->num_leaves == 0) return 0;
-    return (p->items.empty() ? 0 : 1) + 1;                // attention, then merge
+    return (p->items.empty() ? 0 : 1) + (p->direct ? 0 : 1);   // attention, then merge
 }
 
 const char *parason_version(void) { return "0.1.0"; }

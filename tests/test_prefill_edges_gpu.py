@@ -1,0 +1,79 @@
+"""The prefill kernel at its edges: tiles of one row to a pair of full ones
+(32 tokens of 4 q heads are a tile), ancestors that end in every part of a
+128-token block, pages in pool order (one box a block) and permuted (a box a
+page), whole paths that the kernel finishes itself and paths cut into pieces
+that a merge follows."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2608_24658_gb300 import _lib
+from paper_2608_24658_gb300 import workloads as W
+from paper_2608_24658_gb300.api import Plan
+from tests import parity as PT
+
+pytestmark = pytest.mark.gpu
+
+
+def check(tree, whole=None):
+    with Plan.for_prefill(tree) as plan:
+        if whole is not None:
+            assert plan.launches_per_decode() == (1 if whole else 2)
+        out, lse = plan.decode_tree(tree)
+        plan.check()
+    host = tree.to("cpu")
+    kw = oracle.tree_kwargs(host)
+    kw["chunk_node"] = kw.pop("leaf_node")
+    ref_o, ref_l = oracle.prefill(**kw)
+    PT.compare(tree, out, lse, ref_o, ref_l, None, tree.name)
+
+
+@pytest.mark.parametrize("permute", [False, True])
+@pytest.mark.parametrize("mode", ["bf16", "fp8"])
+def test_prefill_tile_and_block_edges(mode, permute):
+    prefixes = [1, 63, 64, 65, 127, 128, 129, 300]
+    chunks = [1, 31, 32, 33, 63, 64, 65, 2]
+    n = len(prefixes)
+    tree = W.build_prefill("edges", [-1] * n + list(range(n)), prefixes + chunks,
+                           list(range(n, 2 * n)), num_q_heads=8, num_kv_heads=2, head_dim=128,
+                           mode=mode, seed=3, permute_pages=permute, extra_pages=5,
+                           tail_value=float("nan"), q_std=0.35, device="cuda")
+    check(tree, whole=mode == "bf16")
+
+
+@pytest.mark.parametrize("mode", ["bf16", "fp8"])
+@pytest.mark.parametrize("g", [1, 5, 8, 16])
+def test_prefill_cut_paths(mode, g):
+    """One chunk over a long chain, more CTAs than pairs: pieces and a merge."""
+    tree = W.build_prefill("cut", [-1, 0, 1, 2], [2500, 70, 1337, 40], [3], num_q_heads=g,
+                           num_kv_heads=1, head_dim=128, mode=mode, seed=4, q_std=0.35,
+                           tail_value=float("nan"), device="cuda")
+    check(tree, whole=False)
+
+
+@pytest.mark.parametrize("mode", ["bf16", "fp8"])
+def test_prefill_growing_maxima(mode):
+    """Keys that grow along the path move the reference max block after block."""
+    tree = W.build_prefill("grow", [-1, 0], [900, 50], [1], num_q_heads=8, num_kv_heads=2,
+                           head_dim=128, mode=mode, seed=5, q_std=0.35, device="cuda")
+    # (a ramp up to 1, with the growth in the scale of q: e4m3 keys already
+    # reach the format's largest value)
+    ramp = torch.linspace(0.03, 1.0, tree.k_pages.shape[0], device="cuda").view(-1, 1, 1, 1)
+    tree.k_pages.copy_((tree.k_pages.float() * ramp).to(tree.k_pages.dtype))
+    tree.q.mul_(3.0)
+    check(tree)
+
+
+def test_prefill_whole_paths_write_the_result():
+    """Without a cut the attention kernel is the only launch; lse may be left out."""
+    tree = W.fork_prefill(device="cuda", chunk=5, threads=3)
+    with Plan.for_prefill(tree) as plan:
+        info = plan.info()
+        mrng = plan.export(_lib.TABLE_MERGE_RANGES)
+        single = bool((mrng[:, 1] - mrng[:, 0] == 1).all())
+        assert plan.launches_per_decode() == (1 if single and info["num_wide_items"] <= 2 * info["num_ctas"] else 2)
+        out, lse = plan.decode_tree(tree)
+        again, none = plan.decode_tree(tree, want_lse=False)
+        plan.check()
+    assert none is None and torch.equal(out, again)
