@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     const uint32_t ring = dev::smem_addr(ring_mem);
     const uint32_t full = dev::smem_addr(bars), empty = full + 8 * NS;
 
+    dev::grid_wait();
     const WorkItem it = a.items[blockIdx.x];
     const int row_groups = (it.nrows + kWarpRows - 1) / kWarpRows;   // 1 .. 4, each a warp's rows
     const int RG = row_groups == 3 ? 4 : row_groups;
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         dev::fence_mbar_init();
     }
     __syncthreads();
-    if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (threadIdx.x == 0) dev::grid_launch_dependents();
 
     // page pg of the item into its stage; pages pg, pg + PG, ... are this
     // warp's, and the warps of row group 0 load them
@@ -332,8 +333,8 @@ cudaError_t launch(const AttnArgs &a, const float *k_pages, const float *v_pages
     const cudaError_t e = cudaFuncSetAttribute(attn_fp32_kernel<D>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, kRing);
     if (e != cudaSuccess) return e;
-    attn_fp32_kernel<D><<<a.num_items, kThreads, kRing, stream>>>(a, k_pages, v_pages);
-    return cudaGetLastError();
+    return launch_dependent(a.early != 0, attn_fp32_kernel<D>, dim3(a.num_items), dim3(kThreads), kRing, stream, a,
+                            k_pages, v_pages);
 }
 
 }  // namespace

@@ -2388,8 +2388,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::fence_before_sync();
     }
     __syncthreads();
-    // let the merge grid launch now; it waits for this grid to complete
-    if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // what precedes in the stream (the last merge, a plan update, whatever made
+    // q, K and V) is complete from here on; then let the merge grid launch, which
+    // waits for this grid to complete
+    dev::grid_wait();
+    if (threadIdx.x == 0) dev::grid_launch_dependents();
 
     if (wide) {
         if constexpr (kTcPrefix) {
@@ -2475,8 +2478,8 @@ cudaError_t launch(const AttnArgs &a, const KvMaps &maps, cudaStream_t stream) {
     using S = Shape<D, KV>;
     cudaError_t e = configure<D, KV>(nullptr);
     if (e != cudaSuccess) return e;
-    attn_kernel<D, KV><<<a.num_ctas, kThreads, S::kSmemBytes, stream>>>(maps, a);
-    return cudaGetLastError();
+    return launch_dependent(a.early != 0, attn_kernel<D, KV>, dim3(a.num_ctas), dim3(kThreads), S::kSmemBytes,
+                            stream, maps, a);
 }
 
 }  // namespace

@@ -100,6 +100,7 @@ struct AttnArgs {
     // no merge runs; out is null otherwise
     void *out;
     float *lse;
+    int32_t early;          // launch as a programmatic dependent (plan.cpp: early)
 };
 
 struct MergeArgs {
@@ -136,6 +137,27 @@ constexpr int kDecodeBoxPages = 1, kPrefillBoxPages = 8;
 struct KvMaps {
     CUtensorMap k, v, k_run, v_run, k_box, v_box;
 };
+
+// Launch, with `early` as a programmatic dependent of the kernel before it in
+// the stream: the CTAs come up (barriers, TMEM, tensor map prefetch) while that kernel
+// drains.  Every kernel launched this way runs griddepcontrol.wait before its
+// first access to global memory; what precedes in the stream is complete and
+// visible from there on.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_dependent(bool early, void (*kernel)(Params...), dim3 grid, dim3 block,
+                                    size_t smem, cudaStream_t stream, Args &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
 
 // Kernel launchers; each returns the launch's cudaError_t.
 cudaError_t launch_attn_bf16(const AttnArgs &a, const KvMaps &maps, int head_dim,

@@ -97,7 +97,9 @@ __global__ void __launch_bounds__(kMergeThreads)
     const int first_e = e0 + w + W * lane;
     const int first_slot = first_e < e1 ? a.merge_ent[first_e] + r : 0;
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    // the attention grid is complete: rewind its work queues for the next call
+    // the attention grid is complete: the next call's may come up (it waits for
+    // this one); rewind the work queues for it
+    if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (blockIdx.x == 0 && threadIdx.x == 0 && a.queue_next) {
         a.queue_next[0] = a.queue_start[0];
         a.queue_next[1] = a.queue_start[1];
@@ -220,7 +222,9 @@ __global__ void __launch_bounds__(kMergeThreads)
     const int e0 = rg.x, e1 = rg.y;
     const int first_slot = e0 + lane < e1 ? a.merge_ent[e0 + lane] : 0;
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    // the attention grid is complete: rewind its work queues for the next call
+    // the attention grid is complete: the next call's may come up (it waits for
+    // this one); rewind the work queues for it
+    if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (blockIdx.x == 0 && threadIdx.x == 0 && a.queue_next) {
         a.queue_next[0] = a.queue_start[0];
         a.queue_next[1] = a.queue_start[1];

@@ -89,6 +89,16 @@ constexpr int64_t kPairShareNum = 3, kPairShareDen = 4;
 // slot even out the launch's end; never longer than kFp32ChunkPages (the
 // fixed length before: 2 to 3 pieces a slot on a 16-branch step).
 constexpr int kFp32ChunkPages = 32;
+// Attention kernels come up while the kernel before them drains (early), which
+// saves a step 2 to 5 us.  Their CTAs then take the SMs in the order these
+// come free, and prefix CTAs and the CTAs that read one kv head are spread
+// less evenly than a launch on an idle GPU spreads them, which costs long
+// launches a share of their time.  Same-box A/B: 16-branch step 34.0 -> 31.2
+// us, two-level 74.2 -> 69.3, 1.5 GB of bf16 KV 243 -> 230, 5.7 GB 834 -> 836;
+// e4m3 KV 0.23 GB 87 -> 84 us, 0.74 GB level, 2.9 GB 517 -> 529; fork prefill
+// (132 pages a CTA) 41.8 -> 39.9 us, join prefill (2150) 524 -> 538.
+constexpr int64_t kEarlyKvBytes = int64_t{2} << 30, kEarlyKvBytesE4m3 = int64_t{3} << 28;
+constexpr int64_t kEarlyPrefillPages = 256;    // a CTA's share
 constexpr int kFp32MinPages = 4;
 constexpr int64_t kFp32Slots = 3, kFp32Waves = 3;
 // stream rows kept free after a branch's last item: half its pages, 4 to 64
@@ -266,6 +276,7 @@ struct parason_plan_s {
     int64_t unique_tokens = 0;
     int64_t path_tokens = 0;
     bool prefill = false;              // a tree-masked prefill plan
+    bool early = false;                // launch while the kernel before drains
     bool direct = false;               // every pair holds its rows' whole paths and has a CTA of
                                        // its own: the attention kernel writes the result
     std::vector<int32_t> shard_branch; // sharded plans: global index of each branch
@@ -978,6 +989,11 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
         if (p->merge_ent.size() > static_cast<size_t>(INT32_MAX)) return PARASON_EUNSUPPORTED;
         p->merge_rng[k] = make_int2(e0, static_cast<int32_t>(p->merge_ent.size()));
     }
+    const int64_t kv_bytes = 2 * p->unique_tokens * H_kv * cfg->head_dim *
+                             (mode == PARASON_FP32 ? 4 : mode == PARASON_BF16 ? 2 : 1);
+    p->early = mode == PARASON_FP32 ||
+               (prefill ? wide_units <= 2 * kEarlyPrefillPages * p->num_sms
+                        : kv_bytes <= (mode == PARASON_BF16 ? kEarlyKvBytes : kEarlyKvBytesE4m3));
     p->direct = prefill && !p->items.empty() &&
                 p->wide_queue.size() <= 2 * static_cast<size_t>(p->num_ctas);
     for (const int2 &rg : p->merge_rng) p->direct = p->direct && rg.y - rg.x == 1;
@@ -1526,6 +1542,7 @@ parason_status parason_attn_decode(parason_plan p, const void *q, const void *k_
         a.item_key0 = p->d_item_key0;
         a.suffix_warps = p->suffix_warps;
         a.tc_pairs = p->tc_pairs ? 1 : 0;
+        a.early = p->early ? 1 : 0;
         if (p->direct) {
             a.out = out;
             a.lse = lse;

@@ -230,8 +230,9 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    // let the merge grid launch now; it waits for this grid to complete
-    if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // (as in attn_kernel)
+    dev::grid_wait();
+    if (threadIdx.x == 0) dev::grid_launch_dependents();
     const uint32_t tmem = tmem_base;
 
     if (warp < 8) {
@@ -848,8 +849,8 @@ template <bool F8, bool DIRECT>
 cudaError_t launch(const AttnArgs &a, const KvMaps &maps, cudaStream_t stream) {
     const cudaError_t e = configure<F8, DIRECT>();
     if (e != cudaSuccess) return e;
-    prefill_kernel<F8, DIRECT><<<a.num_ctas, Cfg<F8>::kThreads, smem_bytes<F8>(), stream>>>(maps, a);
-    return cudaGetLastError();
+    return launch_dependent(a.early != 0, prefill_kernel<F8, DIRECT>, dim3(a.num_ctas),
+                            dim3(Cfg<F8>::kThreads), smem_bytes<F8>(), stream, maps, a);
 }
 
 }  // namespace
