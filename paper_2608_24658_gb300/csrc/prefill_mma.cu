@@ -41,17 +41,19 @@
 // take registers from the others (setmaxnreg; the shares sum to no more than
 // the launch holds).
 //
-// Measured (32 q / 8 kv heads; start of the kernel's own pass to its end):
-// join, 1024 queries over 41k keys, 492 us of 356 us of arithmetic at 1.9
-// PFLOP/s, where the decode kernel's pair tile took 583 us; with e4m3 KV 719 us
-// against 970 us; fork, 16 x 64 queries over 2112 keys, 45 us and no merge
-// against 53 us and a merge.  A pair of blocks takes about 3400 cycles against
-// 2048 of tensor work: a tile's chain is 300 cycles to read S, 400 for the
-// maxima, 1100 for the exponentials, then 768 of its own PV half and S.  Tried
-// and slower: an issuer per tile (both tiles fall into step, 555 -> 727 us),
-// the first half exponentiated before the maxima are known (553 -> 584 us),
-// two threads a row (705 us).  With e4m3 KV the widening warps are the limit:
-// 1100 of about 2550 cycles a slot, the rest spent waiting for slots.
+// Measured (32 q / 8 kv heads, attention kernel): join, 1024 queries over 41k
+// keys, 486 us of 356 us of arithmetic at 1.9 PFLOP/s, where the decode
+// kernel's pair tile took 583 us; with e4m3 KV 730 us against 970 us; fork, 16 x
+// 64 queries over 2112 keys, 45 us and no merge against 53 us and a merge.  A
+// pair of blocks takes about 3400 cycles against 2048 of tensor work: a tile's
+// chain is 300 cycles to read S, 400 for the maxima, 1100 for the
+// exponentials, then 768 of its own PV half and S.  Tried and slower: an issuer
+// per tile (both tiles fall into step, 555 -> 727 us), the first half
+// exponentiated before the maxima are known (553 -> 584 us), two threads a row
+// (705 us).  With e4m3 KV the chain is about 4500 cycles, as the widening warps
+// share the schedulers and the shared memory with the softmax; 8 widening
+// warps (832 us), or widening over the raw bytes in a ring of 5 slots (932
+// us), are slower than a ring of 4 raw and 3 widened slots.
 //
 // Every wait is bounded (%globaltimer); on expiry the error is recorded, the
 // copies in flight land, TMEM is freed and the CTA exits.
@@ -76,6 +78,7 @@ constexpr int kRawSlotBytes = kBlockTokens * 128;              // 16 KB: the sam
 constexpr int kQColBlockBytes = kRows * 128;                   // 16 KB
 constexpr int kQBytes = 2 * kQColBlockBytes;                   // 32 KB a tile
 constexpr int kMeta = 4;
+constexpr int kAheadBlocks = 4;                    // (see the scheduler)
 constexpr int kValidRing = 8;
 constexpr uint32_t kTmemO = 0, kTmemS = 256;
 constexpr int kTmemCols = 512;
@@ -84,9 +87,9 @@ constexpr float kLn2 = 0.69314718055994530942f;
 constexpr int32_t kNoKey0 = -1;                    // the item's rows see all of its keys
 constexpr int kProducerWarp = 8, kMmaWarp = 9, kSchedulerWarp = 10, kConvertWarp = 12;
 
-// Launch shapes.  Registers at launch (threads x the launch bound's share)
-// and after the split: bf16 384 x 168 = 64512 = 256 x 208 + 128 x 88; e4m3
-// 512 x 128 = 65536 = 256 x 176 + 128 x 72 + 128 x 88.
+// Launch shapes, with the registers a thread at launch and after the split:
+// bf16 384 x 168 = 64512 = 256 x 208 + 128 x 88; e4m3 512 x 128 = 65536 = 256 x
+// 152 + 128 x 88 + 128 x 120.
 template <bool F8>
 struct Cfg;
 template <>
@@ -100,7 +103,7 @@ template <>
 struct Cfg<true> {
     static constexpr int kThreads = 512;
     static constexpr int kSlots = 3, kRawSlots = 4;
-    static constexpr int kTileRegs = 176, kAuxRegs = 72, kConvertRegs = 88;
+    static constexpr int kTileRegs = 152, kAuxRegs = 88, kConvertRegs = 120;
     static_assert(256 * kTileRegs + 128 * kAuxRegs + 128 * kConvertRegs <= kThreads * 128,
                   "register split");
 };
@@ -132,8 +135,7 @@ enum Bar : int {
     kOEmpty = kOFull + 2,            // [2] 4 tile warps -> issuer
     kMetaFull = kOEmpty + 2,         // [kMeta] scheduler -> every role
     kMetaEmpty = kMetaFull + kMeta,  // [kMeta] the 8 tile warps -> scheduler
-    kWant = kMetaEmpty + kMeta,      // producer -> scheduler: the next pair
-    kDrain = kWant + 1,              // MMA commit -> issuer, before TMEM is freed
+    kDrain = kMetaEmpty + kMeta,     // MMA commit -> issuer, before TMEM is freed
     kBars
 };
 
@@ -143,7 +145,7 @@ __host__ __device__ constexpr int bar_count(int i, bool f8) {
     if (i >= kSFull && i < kPFull) return 2;
     if (i >= kPFull && i < kOFull) return 4;
     if (i >= kOEmpty && i < kMetaFull) return 4;
-    if (i >= kMetaEmpty && i < kWant) return 8;
+    if (i >= kMetaEmpty && i < kDrain) return 8;
     return 1;
 }
 
@@ -207,6 +209,7 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
     extern __shared__ uint8_t smem_raw[];
     __shared__ int abort_flag;
     __shared__ uint32_t tmem_base;
+    __shared__ volatile int progress;                // pairs the producer is at the end of
     __shared__ int valid_ring[kValidRing];           // valid keys of a block's halves (low bytes)
     __shared__ __align__(8) uint64_t bar_mem[kBars];
     __shared__ Meta meta[kMeta];
@@ -221,6 +224,7 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
+        progress = 0;
         for (int i = 0; i < kBars; ++i) dev::mbar_init(bar(i), bar_count(i, F8));
         dev::fence_mbar_init();
         dev::prefetch_tensormap(&maps.k_box);
@@ -331,10 +335,52 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                     }
                     tc::fence_after_sync();
                     const int vv = valid_ring[(blk + i) % kValidRing];
-                    uint32_t x[4][32];
+                    // The scores: bf16 holds all 128 of the row from here to
+                    // the exponentials; with e4m3 KV, where the converters take
+                    // a third of the registers (and are what the pass waits
+                    // for), each half is read twice.
+                    uint32_t x[F8 ? 2 : 4][32];
+                    auto read_half = [&](int h, uint32_t(&x0)[32], uint32_t(&x1)[32]) {
+                        tc::ld32(tS + 64 * h, x0);
+                        tc::ld32(tS + 64 * h + 32, x1);
+                    };
+                    // keys the row does not see (past the last token of a
+                    // half, or past the row's own token): -inf
+                    const int valid[2] = {vv & 0xff, vv >> 8};
+                    auto hide_half = [&](int h, uint32_t(&x0)[32], uint32_t(&x1)[32]) {
+                        const int seen = min(valid[h], t_rel - (i * kBlockTokens + h * kHalfTokens) + 1);
+                        if (seen < kHalfTokens) {
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) tc::ld32(tS + 32 * c, x[c]);
-                    tc::wait_ld();
+                            for (int q = 0; q < 32; ++q) hide_from(x0[q], q, seen);
+#pragma unroll
+                            for (int q = 0; q < 32; ++q) hide_from(x1[q], q + 32, seen);
+                        }
+                    };
+                    // the max of 64 scores, as two running ones
+                    auto max_half = [](const uint32_t(&x0)[32], const uint32_t(&x1)[32]) {
+                        float m0 = __uint_as_float(x0[0]), m1 = __uint_as_float(x1[0]);
+#pragma unroll
+                        for (int q = 1; q + 1 < 32; q += 2) {
+                            m0 = dev::max3(m0, __uint_as_float(x0[q]), __uint_as_float(x0[q + 1]));
+                            m1 = dev::max3(m1, __uint_as_float(x1[q]), __uint_as_float(x1[q + 1]));
+                        }
+                        return dev::max3(m0, m1, fmaxf(__uint_as_float(x0[31]), __uint_as_float(x1[31])));
+                    };
+                    float mx;
+                    if constexpr (F8) {
+                        read_half(0, x[0], x[1]);
+                        tc::wait_ld();
+                        hide_half(0, x[0], x[1]);
+                        mx = max_half(x[0], x[1]);
+                        read_half(1, x[0], x[1]);
+                        tc::wait_ld();
+                        hide_half(1, x[0], x[1]);
+                        mx = fmaxf(mx, max_half(x[0], x[1]));
+                    } else {
+                        read_half(0, x[0], x[1]);
+                        read_half(1, x[2], x[3]);
+                        tc::wait_ld();
+                    }
                     // the pair's last S is done: the Q buffer takes the next
                     // pair's rows while this block's softmax runs
                     if (i == nb - 1) {
@@ -345,16 +391,10 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                             loaded_next = true;
                         }
                     }
-                    // keys the row does not see (past the last token of a
-                    // half, or past the row's own token): -inf
-                    const int valid[2] = {vv & 0xff, vv >> 8};
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int seen = min(valid[h], t_rel - (i * kBlockTokens + h * kHalfTokens) + 1);
-                        if (seen < kHalfTokens) {
-#pragma unroll
-                            for (int q = 0; q < 64; ++q) hide_from(x[2 * h + (q >> 5)][q & 31], q, seen);
-                        }
+                    if constexpr (!F8) {
+                        hide_half(0, x[0], x[1]);
+                        hide_half(1, x[2], x[3]);
+                        mx = fmaxf(max_half(x[0], x[1]), max_half(x[2], x[3]));
                     }
                     // P of half h as packed 16-bit pairs, against the reference
                     // max m_use (a row that has seen no key: every x is -inf
@@ -364,7 +404,7 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                         const unsigned long long nmp = dev::f32x2(-m_ref, -m_ref);
 #pragma unroll
                         for (int c = 0; c < 32; ++c) {
-                            const uint32_t(&xc)[32] = x[2 * h + (c >> 4)];
+                            const uint32_t(&xc)[32] = x[(F8 ? 0 : 2 * h) + (c >> 4)];
                             float e0, e1;
                             dev::f32x2_split(
                                 dev::fma_f32x2(dev::f32x2(__uint_as_float(xc[2 * (c & 15)]),
@@ -379,17 +419,6 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                     };
                     uint32_t pw[32];
                     unsigned long long lsum = 0ull;
-                    float mr[4];
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        mr[c] = __uint_as_float(x[c][0]);
-#pragma unroll
-                        for (int q = 1; q + 1 < 32; q += 2)
-                            mr[c] = dev::max3(mr[c], __uint_as_float(x[c][q]), __uint_as_float(x[c][q + 1]));
-                    }
-                    float mx = dev::max3(mr[0], mr[1], fmaxf(mr[2], mr[3]));
-                    mx = fmaxf(mx, dev::max3(__uint_as_float(x[0][31]), __uint_as_float(x[1][31]),
-                                             fmaxf(__uint_as_float(x[2][31]), __uint_as_float(x[3][31]))));
                     const float mb = mx * sl;
                     if (i == 0) {
                         m_use = mb;
@@ -413,6 +442,11 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                     }
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
+                        if constexpr (F8) {
+                            read_half(h, x[0], x[1]);
+                            tc::wait_ld();
+                            hide_half(h, x[0], x[1]);
+                        }
                         lsum = exponentiate(h, pw, lsum);
                         tc::st32(tS + 32 * h, pw);
                         // V rows past the half's valid tokens may hold anything
@@ -551,12 +585,35 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
         reg_dec<C::kAuxRegs>();
         if (warp == kSchedulerWarp) {
             // -------------------------------------------------------- scheduler
+            int nbs[kMeta] = {0, 0, 0, 0};                  // blocks of the last pairs
+            auto reached = [&](int pairs) {
+                int there = 1;
+                if (lane == 0 && progress < pairs) {
+                    const uint64_t t0 = dev::global_timer_ns();
+                    while (progress < pairs) {
+                        if (*abort || static_cast<long long>(dev::global_timer_ns() - t0) > limit) {
+                            there = 0;
+                            break;
+                        }
+                        __nanosleep(100);
+                    }
+                }
+                return __shfl_sync(0xffffffffu, there, 0) != 0;
+            };
             for (int k = 0;; ++k) {
                 const int s = k % kMeta;
-                // A pair is pulled once the producer is at the last block of the
-                // one before (a CTA that pulled as soon as a slot was free took
-                // pairs that others had time for: join prefill kernel 553 -> 492 us)
-                if ((k > 0 && !tc_warp_wait(bar(kWant), (k - 1) & 1, limit, abort, lane)) ||
+                // A pair is pulled once the producer is near the end of the one
+                // before (a CTA that pulled as soon as a slot was free took
+                // pairs that others had time for: join prefill kernel 553 ->
+                // 492 us); pairs of a few blocks are pulled up to kMeta ahead,
+                // while together they are no more than kAheadBlocks, so that
+                // their records' latency does not add up.
+                int need = k;                              // pairs the producer has to be through
+                for (int ahead = 0; need > 0 && k - need < kMeta - 1; --need) {
+                    ahead += nbs[(need - 1) % kMeta];
+                    if (ahead > kAheadBlocks) break;
+                }
+                if (!reached(need) ||
                     (k >= kMeta &&
                      !tc_warp_wait(bar(kMetaEmpty + s), ((k / kMeta) - 1) & 1, limit, abort, lane))) {
                     if (lane == 0) tc_fail(a, abort, kSiteProducerEmpty);
@@ -600,6 +657,8 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                     dev::mbar_arrive(bar(kMetaFull + s));
                 }
                 if (__shfl_sync(0xffffffffu, id, 0) < 0) break;
+                __syncwarp();
+                nbs[s] = blocks_of(meta[s].it.num_pages);
             }
         } else if (warp == kProducerWarp) {
             // -------------------------------------------------------- producer
@@ -638,7 +697,7 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                 int32_t next = rows[lane], win = 0;
                 uint32_t ends = 0, follows = 0, pool = 0;
                 for (int i = 0; i < nb && ok; ++i, ++blk) {
-                    if (i == nb - 1 && lane == 0) dev::mbar_arrive(bar(kWant));
+                    if (i == max(0, nb - 2) && lane == 0) progress = k + 1;
                     const int pg0 = i * kBlockPages, w0 = pg0 & 31;
                     if (w0 == 0) {
                         // past the item: the first row past the pool, which TMA
