@@ -9,7 +9,7 @@
 //    into one tile against the node's pages, so the node's KV is read from
 //    HBM once for all of them, which is what the shared prefix of
 //    Subtask/Trial branches buys (paper Sec. 3.1, 3.4).
-//      - head_dim 128 (bf16 or e4m3 KV): a tcgen05 tile (prefix_cta_tc).
+//      - a tcgen05 tile (prefix_cta_tc; bf16 at both head dims, e4m3 KV).
 //        Warp roles: a scheduler warp stages each item's metadata; a
 //        producer warp moves 64-token blocks of K and V by TMA (one 5-D box
 //        per column block when the block's 4 pages are consecutive in the
@@ -24,9 +24,6 @@
 //        128-row tiles of a piece against each staged block
 //        (prefix_cta_tc_pair), Q in shared memory, each tile's S/P and O in
 //        TMEM, so that a block is staged once for 256 rows.
-//      - head_dim 64: mma.sync (prefix_cta): a producer warp streams pages
-//        into a ring, 8 consumer warps of 16 rows share the pages and combine
-//        through shared memory.
 //  * suffix pass (the other CTAs, and prefix CTAs once the prefix queue is
 //    empty): nodes of at most 16 rows (a branch's own suffix).  Each warp is
 //    an independent worker with its own TMA ring that pulls split-K pieces
@@ -64,17 +61,13 @@
 namespace parason {
 namespace {
 
-constexpr int kConsumerWarps = 8;                          // prefix pass on mma.sync
-constexpr int kConsumerThreads = kConsumerWarps * 32;
 constexpr int kMaxSuffixWarps = 12;                        // suffix pass: warps per CTA, at most
 // 12 warps: the suffix pass runs 6, 8 or 12 autonomous warps (by KV type);
-// the prefix pass on tcgen05 uses all 12 (softmax 4, epilogue 4, producer,
-// S issuer, scheduler, PV issuer), the one on mma.sync 9 (8 consumers and a
-// producer)
+// the prefix pass uses all 12 (softmax 4, epilogue 4, producer, S issuer,
+// scheduler, PV issuer)
 constexpr int kThreads = 12 * 32;
 constexpr long long kDrainLimitNs = 1000000000LL;
 constexpr int kSmemBudget = 220 * 1024;                    // dynamic, one CTA per SM
-constexpr int kIdSlots = 8;      // prefix-pass item ids in flight from producer to consumers
 constexpr int kGrabSlots = 8;    // suffix-pass item ids a warp has pulled but not finished
 constexpr float kLazyRescaleLog2 = 8.f;   // mma.sync softmax: move the reference max past 2^8
 
@@ -119,47 +112,21 @@ struct Shape {
     static constexpr int kNarrowBytes = kSuffixWarps * kWarpRingBytes;
     static constexpr int kNarrowBars = kSuffixWarps * kWarpStages;
 
-    // prefix pass: one ring + combine scratch [warp][16 rows][D/2 + 8] floats
-    static constexpr int kHalf = D / 2;
-    static constexpr int kScratchStride = kHalf + 8;
-    static constexpr int kScratchBytes = kConsumerWarps * 16 * (kScratchStride * 4 + 8);
-    static constexpr int kWideStages = (kNarrowBytes - kScratchBytes) / kStageBytes;
-    static constexpr int kWideRingBytes = kWideStages * kStageBytes;
-    static constexpr int kWideBars = 2 * kWideStages;
-
-    // + kIdSlots item-id barriers of the prefix pass, + the tcgen05 tile's 16
-    static constexpr int kWideAll = kWideBars + kIdSlots;
-    static constexpr int kBars0 = kNarrowBars > kWideAll ? kNarrowBars : kWideAll;
-    static constexpr int kBars = kBars0 > 16 + kIdSlots ? kBars0 : 16 + kIdSlots;
-    static constexpr int kBodyBytes =
-        kNarrowBytes > kWideRingBytes + kScratchBytes ? kNarrowBytes : kWideRingBytes + kScratchBytes;
+    static constexpr int kBars = 64;                        // the larger of both passes' barriers
+    static constexpr int kBodyBytes = kNarrowBytes;
     static constexpr int kSmemBytes = kBodyBytes + kBars * 8 + 1024;   // + alignment slack
+    static_assert(kNarrowBars <= kBars, "barrier area holds the suffix rings' barriers");
     static_assert(kRowBytes % 128 == 0, "token rows are whole 128-byte blocks");
     static_assert(kWarpStages >= 2, "suffix ring depth");
     static_assert(kSuffixWarps <= kMaxSuffixWarps, "suffix-pass warps fit the item rings");
-    static_assert(kWideStages >= 4, "prefix ring depth");
     static_assert(kSmemBytes <= kSmemBudget, "shared memory budget");
 
 };
 
-// K then V of one (page, kv head) into a stage: one TMA box {128 bytes, 1
-// block, 16 tokens} per column block and tensor (the prefix pass of the
-// mma.sync path; a prefix page may be read again by another row tile of its
-// node and keeps the normal L2 policy).
-template <int D, class KV>
-__device__ __forceinline__ void load_page(uint32_t dst, const CUtensorMap *tmap_k,
-                                          const CUtensorMap *tmap_v, int row, uint32_t bar) {
-    using S = Shape<D, KV>;
-#pragma unroll
-    for (int sg = 0; sg < S::kSeg; ++sg) {
-        dev::tma_load_3d(dst + sg * S::kSegBytes, tmap_k, 0, sg, row, bar);
-        dev::tma_load_3d(dst + S::kPageBytes + sg * S::kSegBytes, tmap_v, 0, sg, row, bar);
-    }
-}
-
-// The same for a suffix page, in one box per tensor (the page maps) where a
-// page has several column blocks: half the copies at head_dim 128 bf16, in
-// the same shared-memory layout (same-box A/B: two-level step 81.8 -> 79.6
+// K then V of one (page, kv head) into a suffix stage, in one TMA box per
+// tensor (the page maps) where a page has several column blocks: half the
+// copies at head_dim 128 bf16 of a box per block, in the same shared-memory
+// layout (same-box A/B: two-level step 81.8 -> 79.6
 // us, long prefix 839.6 -> 834.2 us).  A suffix page is read by one item
 // only, so its lines go first when L2 needs room (the partials written
 // meanwhile stay for the merge).
@@ -732,26 +699,6 @@ __device__ __forceinline__ int pull(const AttnArgs &a, int which, int lane) {
     return __shfl_sync(0xffffffffu, id, 0);
 }
 
-// The TMA rows of one item's pages, read by one whole warp 32 at a time: lane
-// i holds row base + i; row(pg) returns the row of page pg (pg uniform over
-// the warp, nondecreasing within an item).
-struct ItemRows {
-    const int32_t *rows = nullptr;
-    int base = -1;
-    int win = 0;
-    __device__ void start(const AttnArgs &a, int item) {
-        rows = a.stream_rows + a.item_rows[item];
-        base = -1;
-    }
-    __device__ __forceinline__ int row(int pg, int lane) {
-        if (base < 0 || pg >= base + 32) {
-            base = pg & ~31;
-            win = rows[base + lane];        // the row array is padded by 32 entries
-        }
-        return __shfl_sync(0xffffffffu, win, pg - base);
-    }
-};
-
 // ---------------------------------------------------------------------------
 // suffix pass: every warp pulls items from the suffix queue and streams their
 // pages through its own ring
@@ -918,201 +865,8 @@ __device__ void suffix_warp(const KvMaps &maps, const AttnArgs &a, uint32_t ring
     __syncwarp();
 }
 
-// Prefix pass: the producer warp pulls items and hands their ids to the
-// consumer warps through kIdSlots shared slots, each with an mbarrier (id -1
-// ends the queue).  The producer is never more than a few items ahead of the
-// slowest consumer (it waits for ring stages they release), so the slots
-// are never overwritten before they are read.
-__device__ __forceinline__ void publish_id(volatile int *slots, uint32_t id_bars, int k, int id) {
-    slots[k % kIdSlots] = id;
-    dev::mbar_arrive(id_bars + 8 * (k % kIdSlots));
-}
-
-__device__ __forceinline__ int take_id(const volatile int *slots, uint32_t id_bars, int k,
-                                       long long limit, volatile int *abort, bool *ok) {
-    if (!dev::mbar_wait_bounded(id_bars + 8 * (k % kIdSlots), (k / kIdSlots) & 1, limit, abort)) {
-        *ok = false;
-        return -1;
-    }
-    return slots[k % kIdSlots];
-}
-
 // ---------------------------------------------------------------------------
-// prefix pass: up to 128 stacked rows share one page stream
-// ---------------------------------------------------------------------------
-template <int D, class KV>
-__device__ void prefix_cta(const CUtensorMap *tmap_k, const CUtensorMap *tmap_v,
-                           const AttnArgs &a, uint8_t *smem, uint32_t ring, uint32_t bars,
-                           int warp, int lane, volatile int *abort_flag, volatile int *id_slots) {
-    using S = Shape<D, KV>;
-    constexpr int NS = S::kWideStages;
-    const uint32_t bar_full = bars, bar_empty = bars + NS * 8;
-    const uint32_t id_bars = bars + 2 * NS * 8;
-    auto k_page = [&](int s) { return ring + s * S::kStageBytes; };
-
-    if (warp == kConsumerWarps) {
-        // ------------------------------------------------------------ producer
-        // the whole warp pulls items and walks their pages; lane 0 waits and issues
-        int last_issue[NS];
-        for (int s = 0; s < NS; ++s) last_issue[s] = -1;
-        const bool skip_first = a.debug_flags & PARASON_DEBUG_SKIP_FIRST_LOAD;
-        int stage = 0;
-        bool go = true;
-        for (int k = 0; go; ++k) {
-            // a prefix CTA owns position blockIdx.x of the prefix queue
-            const int id = *abort_flag ? -1
-                                       : (k == 0 ? queue_item(a, 0, static_cast<int>(blockIdx.x))
-                                                 : pull(a, 0, lane));
-            if (lane == 0) publish_id(id_slots, id_bars, k, id);
-            if (id < 0) break;
-            ItemRows rows;
-            rows.start(a, id);
-            const int np = a.items[id].num_pages;
-            for (int pg = 0; pg < np; ++pg, ++stage) {
-                const int s = stage % NS;
-                int stop = 0;
-                if (lane == 0) {
-                    if (stage >= NS && !dev::mbar_wait_bounded(bar_empty + 8 * s,
-                                                               ((stage / NS) - 1) & 1,
-                                                               a.wait_limit_ns, abort_flag)) {
-                        if (!*abort_flag) {
-                            *abort_flag = 1;
-                            dev::record_error(a.err, PARASON_ETIMEOUT, kSiteProducerEmpty);
-                        }
-                        stop = 1;
-                    } else if (*abort_flag) {
-                        stop = 1;
-                    }
-                }
-                if (__shfl_sync(0xffffffffu, stop, 0)) {
-                    go = false;
-                    break;
-                }
-                const int row = rows.row(pg, lane);
-                if (lane == 0 && !(skip_first && stage == 0)) {
-                    dev::mbar_arrive_expect_tx(bar_full + 8 * s, S::kStageBytes);
-                    load_page<D, KV>(k_page(s), tmap_k, tmap_v, row, bar_full + 8 * s);
-                    last_issue[s] = stage;
-                }
-            }
-        }
-        // every copy this CTA issued must land before its shared memory goes
-        if (lane == 0)
-            for (int s = 0; s < NS; ++s)
-                if (last_issue[s] >= 0)
-                    dev::mbar_wait_bounded(bar_full + 8 * s, (last_issue[s] / NS) & 1, kDrainLimitNs,
-                                           nullptr);
-        return;
-    }
-    if (warp > kConsumerWarps) return;
-
-    // ---------------------------------------------------------------- consumers
-    uint8_t *scratch = smem + S::kWideRingBytes;
-    float *sc_o = reinterpret_cast<float *>(scratch);
-    float2 *sc_ml = reinterpret_cast<float2 *>(scratch + kConsumerWarps * 16 * S::kScratchStride * 4);
-    const int tid = threadIdx.x;
-    const int gid = lane >> 2, tig = lane & 3;
-    int stage = 0;
-    for (int k = 0;; ++k) {
-        bool got = true;
-        const int id = take_id(id_slots, id_bars, k, a.wait_limit_ns, abort_flag, &got);
-        if (dev::bar_sync_or<kConsumerThreads>(1, !got || id < 0)) break;
-        const WorkItem it = a.items[id];
-        const float2 scl = item_scales<KV>(a, it);
-        const int groups = (it.nrows + 15) >> 4;
-        const int rgc = groups <= 2 ? 2 : (groups <= 4 ? 4 : 8);
-        const int tgc = kConsumerWarps / rgc;
-        const int rg = warp / tgc, tg = warp % tgc;
-        const bool has_rows = rg * 16 < it.nrows;
-
-        uint32_t qa[D / 16][4];
-        load_q_fragments<D, KV>(a, it, rg, lane, qa);
-        WarpState<D> st;
-        reset<D>(st);
-
-        // page pg goes to token-group warp pg % tgc of each row group; every
-        // warp waits for every page (keeping the empty barrier's phases exact)
-        // and releases it
-        bool ok = true;
-        for (int pg = 0; pg < it.num_pages; ++pg, ++stage) {
-            const int s = stage % NS;
-            if (!dev::mbar_wait_bounded(bar_full + 8 * s, (stage / NS) & 1, a.wait_limit_ns,
-                                        abort_flag)) {
-                ok = false;
-                break;
-            }
-            if (has_rows && pg % tgc == tg) {
-                const int valid = (pg == it.num_pages - 1) ? it.last_valid : kPageSize;
-                page_step<D, KV>(k_page(s), k_page(s) + S::kPageBytes, valid, qa, st, scl.x, lane);
-            }
-            __syncwarp();
-            if (lane == 0) dev::mbar_arrive(bar_empty + 8 * s);
-        }
-        if (!ok && lane == 0 && !*abort_flag) {
-            *abort_flag = 1;
-            dev::record_error(a.err, PARASON_ETIMEOUT, kSiteConsumerFull);
-        }
-        // one decision for all consumer warps, whatever the producer does meanwhile
-        if (dev::bar_sync_or<kConsumerThreads>(1, !ok || *abort_flag)) break;
-
-        if (tgc == 1) {
-            if (has_rows) store_warp_partials<D, KV>(a, it, st, rg, lane, scl.y);
-            continue;
-        }
-        // combine the token-group warps of each row group, one column half at a time
-        st.l[0] += __shfl_xor_sync(0xffffffffu, st.l[0], 1);
-        st.l[0] += __shfl_xor_sync(0xffffffffu, st.l[0], 2);
-        st.l[1] += __shfl_xor_sync(0xffffffffu, st.l[1], 1);
-        st.l[1] += __shfl_xor_sync(0xffffffffu, st.l[1], 2);
-        if (tig == 0) {
-            sc_ml[warp * 16 + gid] = make_float2(st.m[0], st.l[0]);
-            sc_ml[warp * 16 + gid + 8] = make_float2(st.m[1], st.l[1]);
-        }
-        constexpr int kVec = S::kHalf / 4;
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            float *wo = sc_o + warp * 16 * S::kScratchStride;
-#pragma unroll
-            for (int dt = 0; dt < D / 8; ++dt)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int col = out_col<KV>(dt, e, tig);
-                    if (col / S::kHalf == half)
-                        wo[(gid + 8 * (e >> 1)) * S::kScratchStride + col % S::kHalf] =
-                            st.o[dt][e] * scl.y;
-                }
-            dev::bar_sync<kConsumerThreads>(1);
-            for (int idx = tid; idx < it.nrows * kVec; idx += kConsumerThreads) {
-                const int r = idx / kVec, c4 = idx % kVec;
-                const int grp = r >> 4, rr = r & 15;
-                float M = -INFINITY;
-                for (int w = 0; w < tgc; ++w) M = fmaxf(M, sc_ml[(grp * tgc + w) * 16 + rr].x);
-                float L = 0.f;
-                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int w = 0; w < tgc; ++w) {
-                    const int ww = grp * tgc + w;
-                    const float2 ml = sc_ml[ww * 16 + rr];
-                    const float sc = dev::fast_exp2(ml.x - M);
-                    L += sc * ml.y;
-                    const float4 v = *reinterpret_cast<const float4 *>(
-                        sc_o + (ww * 16 + rr) * S::kScratchStride + 4 * c4);
-                    acc.x += sc * v.x;
-                    acc.y += sc * v.y;
-                    acc.z += sc * v.z;
-                    acc.w += sc * v.w;
-                }
-                const int64_t slot = static_cast<int64_t>(it.slot_base) + r;
-                *reinterpret_cast<float4 *>(a.part_o + slot * D + half * S::kHalf + 4 * c4) = acc;
-                if (half == 0 && c4 == 0) a.part_ml[slot] = make_float2(M, L);
-            }
-            dev::bar_sync<kConsumerThreads>(1);
-        }
-    }
-}
-
-
-// ---------------------------------------------------------------------------
-// prefix pass on tcgen05 (bf16 or e4m3 KV, head_dim 128): a tile of up to 128
+// prefix pass on tcgen05 (bf16 KV, e4m3 KV at head_dim 128): a tile of up to 128
 // stacked rows against 64-token blocks (4 pages) of the node's pages
 //
 //   warp 10     scheduler: pulls items from the prefix queue and stages each
@@ -1141,6 +895,11 @@ __device__ void prefix_cta(const CUtensorMap *tmap_k, const CUtensorMap *tmap_v,
 //               partials and loads the Q rows of the item two ahead into the
 //               TMEM Q buffer that item frees (Q of items 0 and 1 at start);
 //               with e4m3 KV they also convert every staged block to f16
+//
+// At head_dim 64 a stage is 16 KB and every product half as deep or as wide
+// (against a prefix pass on mma.sync, 8 warps of 16 rows page by page: 4 requests
+// x 32 branches over 2k to 8k prefixes 66.4 -> 42.8 us, 16k prefix and 64
+// branches of 8 heads 199 -> 87.8 us).
 //
 // TMEM, 512 columns: O[2] at 0 and 128, S/P[2] at 256 and 320, Q[2] at 384
 // and 448.  Shared memory: the ring [6][K: 2 col blocks x 64 tokens x 128 B |
@@ -1287,8 +1046,12 @@ template <int D, class KV>
 __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *smem, uint32_t bars,
                               uint32_t tmem, int warp, int lane, volatile int *abort_flag,
                               TcMeta *meta) {
-    static_assert(D == 128, "the tcgen05 prefix tile is written for head_dim 128");
     constexpr bool kF8 = KV::kElemBytes == 1;
+    static_assert(D == 128 || (D == 64 && !kF8), "head_dim 128, or 64 with bf16 KV");
+    constexpr int kCols = D / 64;                        // 64-element column blocks of K (of V)
+    constexpr int kKBytes = kCols * kTcColBlockBytes;
+    constexpr int kStageBytes = 2 * kKBytes;
+    static_assert(kTcStages * kStageBytes <= Shape<D, KV>::kBodyBytes, "ring fits the CTA's memory");
     const uint32_t ring = dev::smem_addr(smem);
     auto bar = [&](int i) { return bars + 8u * static_cast<uint32_t>(i); };
     const long long limit = a.wait_limit_ns;
@@ -1369,7 +1132,7 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                     // expected bytes are registered first
                     const uint32_t fb = bar(kBarKvFull + s);
                     if (lane == 0)
-                        dev::mbar_arrive_expect_tx(fb, kF8 ? kTcF8StageBytes : kTcStageBytes);
+                        dev::mbar_arrive_expect_tx(fb, kF8 ? kTcF8StageBytes : kStageBytes);
                     __syncwarp();
                     // the TMA unit takes about 90 cycles a box, so a block of
                     // pages that are consecutive in the pool (the common case)
@@ -1389,8 +1152,8 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                                                       m.it.kv_head, page, fb, f8_pol);
                         } else {
                             // lane: K (even) or V, column block lane / 2
-                            if (lane < 4)
-                                dev::tma_load_5d_hint(ring + s * kTcStageBytes + (lane & 1) * kTcKBytes +
+                            if (lane < 2 * kCols)
+                                dev::tma_load_5d_hint(ring + s * kStageBytes + (lane & 1) * kKBytes +
                                                           (lane >> 1) * kTcColBlockBytes,
                                                       (lane & 1) ? &maps->v_run : &maps->k_run, 0,
                                                       lane >> 1, 0, m.it.kv_head, page, fb, last_pol);
@@ -1406,13 +1169,13 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                                              0, 0, row, fb);
                         }
                     } else {
-                        // page j = lane / 4, column block (lane / 2) % 2, K (even lanes) or V
-                        if (lane < 4 * kTcBlockPages) {
-                            const int j = lane >> 2, cb = (lane >> 1) & 1;
+                        // page j, column block cb, K (even lanes) or V
+                        if (lane < 2 * kCols * kTcBlockPages) {
+                            const int j = lane / (2 * kCols), cb = (lane >> 1) % kCols;
                             const int pg = bi * kTcBlockPages + j;
                             const int row = pg < np ? m.rows[pg] : a.kv_rows;   // kv_rows: zero fill
                             const uint32_t off = cb * kTcColBlockBytes + j * kPageSize * 128;
-                            const uint32_t st = ring + s * kTcStageBytes + (lane & 1) * kTcKBytes;
+                            const uint32_t st = ring + s * kStageBytes + (lane & 1) * kKBytes;
                             dev::tma_load_3d_hint(st + off, (lane & 1) ? &maps->v : &maps->k, 0, cb,
                                                   row, fb, last_pol);
                         }
@@ -1456,8 +1219,8 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
             // the start address field (address / 16) by a constant
             const uint32_t mma_ring = kF8 ? ring + kTcCvOffset : ring;
             const uint64_t desc_k = tc::smem_desc_sw128(mma_ring, 16, 1024);
-            const uint64_t desc_v = tc::smem_desc_sw128(mma_ring + kTcKBytes, kTcColBlockBytes, 1024);
-            constexpr uint32_t kStageStep = kTcStageBytes >> 4;
+            const uint64_t desc_v = tc::smem_desc_sw128(mma_ring + kKBytes, kTcColBlockBytes, 1024);
+            constexpr uint32_t kStageStep = kStageBytes >> 4;
             int b = 0;                       // block of the CTA's stream
             int st = 0, ph = 0;              // its stage and the stage's phase parity
             for (int k = 0;; ++k) {
@@ -1620,10 +1383,10 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                 // included); P is 0 there but 0 * NaN is NaN, so zero them (the
                 // e4m3 converters write those rows as zeros)
                 if (!kF8 && valid < kTcBlockTokens) {
-                    const uint32_t vst = ring + (b % kTcStages) * kTcStageBytes + kTcKBytes;
-                    const int n16 = (kTcBlockTokens - valid) * 2 * 8;     // 16-byte chunks
+                    const uint32_t vst = ring + (b % kTcStages) * kStageBytes + kKBytes;
+                    const int n16 = (kTcBlockTokens - valid) * kCols * 8;     // 16-byte chunks
                     for (int q = r; q < n16; q += kTcRows) {
-                        const int t = valid + q / 16, cb = (q / 8) & 1, c = q & 7;
+                        const int t = valid + q / (8 * kCols), cb = (q / 8) % kCols, c = q & 7;
                         asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(
                                          vst + cb * kTcColBlockBytes + t * 128 + (c << 4)),
                                      "r"(0u)
@@ -1657,7 +1420,7 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
             return meta[k % kTcMeta].id >= 0;
         };
         // Q row r of item k: global loads into registers ...
-        auto fetch_q = [&](int k, uint4 (&qv)[16]) {
+        auto fetch_q = [&](int k, uint4 (&qv)[D / 8]) {
             const TcMeta &m = meta[k % kTcMeta];
             if (r < m.it.nrows) {
                 const int leaf = m.leaves[r / a.group];
@@ -1666,22 +1429,22 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                     static_cast<const __nv_bfloat16 *>(a.q) +
                     (static_cast<int64_t>(leaf) * a.num_q_heads + head) * D);
 #pragma unroll
-                for (int c = 0; c < 16; ++c) qv[c] = src[c];
+                for (int c = 0; c < D / 8; ++c) qv[c] = src[c];
             } else {
 #pragma unroll
-                for (int c = 0; c < 16; ++c) qv[c] = make_uint4(0u, 0u, 0u, 0u);
+                for (int c = 0; c < D / 8; ++c) qv[c] = make_uint4(0u, 0u, 0u, 0u);
             }
         };
         // ... then into TMEM Q buffer k & 1 (bf16 pairs, or f16 pairs for
         // the e4m3 tile, lane r)
-        auto put_q = [&](int k, const uint4 (&qv)[16]) {
+        auto put_q = [&](int k, const uint4 (&qv)[D / 8]) {
             bool big = false;
             auto cv = [&big](uint32_t two) {
                 if constexpr (!kF8) return two;
                 return q_pair_to_f16(two, big);
             };
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int h = 0; h < D / 64; ++h) {
                 uint32_t w[32];
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
@@ -1726,7 +1489,7 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                     !tc_warp_wait(bar(kBarCvEmpty + c), ((gb / kTcCvStages) - 1) & 1, limit, abort_flag,
                                   lane))
                     return false;
-                convert_block_e4m3(ring + s * kTcF8StageBytes, ring + kTcCvOffset + c * kTcStageBytes,
+                convert_block_e4m3(ring + s * kTcF8StageBytes, ring + kTcCvOffset + c * kStageBytes,
                                    valid, r);
                 tc::fence_proxy_async_smem();
                 dev::mbar_arrive(bar(kBarCvFull + c));
@@ -1742,7 +1505,7 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                 tc::fence_after_sync();
                 const bool has_j2 = next_exists && has_item(j + 2);
                 if (!ok) return false;
-                uint4 qv[16];
+                uint4 qv[D / 8];
                 if (has_j2) fetch_q(j + 2, qv);
                 store_o(j, it);
                 if (has_j2) put_q(j + 2, qv);
@@ -1755,7 +1518,7 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                 return true;
             };
             if (has_item(0)) {
-                uint4 qv[16];
+                uint4 qv[D / 8];
                 fetch_q(0, qv);
                 put_q(0, qv);
                 if (has_item(1)) {
@@ -1784,7 +1547,7 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
         }
         bool has_k = has_item(0), has_k1 = false;
         if (has_k) {
-            uint4 qv[16];
+            uint4 qv[D / 8];
             fetch_q(0, qv);
             put_q(0, qv);
             has_k1 = has_item(1);
@@ -1803,7 +1566,7 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
             // item k's S MMAs are complete, so its Q buffer takes item k + 2's rows;
             // their loads are in flight while O is stored
             const bool has_k2 = has_k1 && has_item(k + 2);
-            uint4 qv[16];
+            uint4 qv[D / 8];
             if (has_k2) fetch_q(k + 2, qv);
             const uint32_t tO = lane_base + kTmemO + 128u * (k & 1);
             float *dst = a.part_o + (static_cast<int64_t>(it.slot_base) + r) * D;
@@ -2343,35 +2106,26 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t ring = dev::smem_addr(smem);
     const uint32_t bars = dev::smem_addr(smem + S::kBodyBytes);
     __shared__ int abort_flag;
-    __shared__ int id_slots[kIdSlots];                        // prefix-pass item ids
     __shared__ WorkItem grab_items[kMaxSuffixWarps][kGrabSlots];  // suffix-pass items per warp
     const bool wide = static_cast<int>(blockIdx.x) < a.num_wide_ctas;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    // the prefix pass at head_dim 128 (bf16 or e4m3 KV) runs on tcgen05; with
-    // bf16 KV the plan may hand it pairs of row tiles (pair mode)
-    constexpr bool kTcPrefix = D == 128;
-    const bool tc_pairs = kTcPrefix && KV::kElemBytes == 2 && a.tc_pairs != 0;
-    const int prefix_bars =
-        kTcPrefix ? (tc_pairs ? static_cast<int>(kTcPairBars) : static_cast<int>(kTcBars))
-                  : 2 * S::kWideStages + kIdSlots;
-    static_assert(!kTcPrefix || (kTcBars <= S::kBars && kTcPairBars <= S::kBars),
+    // with bf16 KV at head_dim 128 the plan may hand the prefix pass pairs of
+    // row tiles (pair mode)
+    constexpr bool kPairs = D == 128 && KV::kElemBytes == 2;
+    const bool tc_pairs = kPairs && a.tc_pairs != 0;
+    const int prefix_bars = tc_pairs ? static_cast<int>(kTcPairBars) : static_cast<int>(kTcBars);
+    static_assert(kTcBars <= S::kBars && kTcPairBars <= S::kBars,
                   "barrier area holds the tcgen05 barriers");
-    __shared__ TcMeta tc_meta[kTcPrefix ? kTcMeta : 1];
+    __shared__ TcMeta tc_meta[kTcMeta];
     __shared__ uint32_t tmem_base;
     if (threadIdx.x == 0) {
         abort_flag = 0;
-        if (wide && kTcPrefix && tc_pairs) {
+        if (wide && tc_pairs) {
             for (int i = 0; i < kTcPairBars; ++i) dev::mbar_init(bars + 8 * i, tc_pair_bar_count(i));
-        } else if (wide && kTcPrefix) {
+        } else if (wide) {
             for (int i = 0; i < kTcBars; ++i)
                 dev::mbar_init(bars + 8 * i, tc_bar_count(i, KV::kElemBytes == 1));
-        } else if (wide) {
-            for (int s = 0; s < S::kWideStages; ++s) {
-                dev::mbar_init(bars + 8 * s, 1);
-                dev::mbar_init(bars + 8 * (S::kWideStages + s), kConsumerWarps);
-            }
-            for (int i = 0; i < kIdSlots; ++i) dev::mbar_init(bars + 8 * (2 * S::kWideStages + i), 1);
         } else {
             for (int s = 0; s < S::kNarrowBars; ++s) dev::mbar_init(bars + 8 * s, 1);
         }
@@ -2383,10 +2137,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             dev::prefetch_tensormap(&maps.v_box);
         }
     }
-    if constexpr (kTcPrefix) {
-        if (wide && warp == kTcMmaWarp) tc::alloc<kTcTmemCols>(dev::smem_addr(&tmem_base));
-        tc::fence_before_sync();
-    }
+    if (wide && warp == kTcMmaWarp) tc::alloc<kTcTmemCols>(dev::smem_addr(&tmem_base));
+    tc::fence_before_sync();
     __syncthreads();
     // what precedes in the stream (the last merge, a plan update, whatever made
     // q, K and V) is complete from here on; then let the merge grid launch, which
@@ -2395,27 +2147,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (threadIdx.x == 0) dev::grid_launch_dependents();
 
     if (wide) {
-        if constexpr (kTcPrefix) {
-            tc::fence_after_sync();
-            if constexpr (KV::kElemBytes == 2) {
-                if (tc_pairs)
-                    prefix_cta_tc_pair<D>(&maps, a, smem, bars, tmem_base, warp, lane, &abort_flag,
-                                          tc_meta);
-                else
-                    prefix_cta_tc<D, KV>(&maps, a, smem, bars, tmem_base, warp, lane, &abort_flag,
-                                         tc_meta);
-            } else {
-                prefix_cta_tc<D, KV>(&maps, a, smem, bars, tmem_base, warp, lane, &abort_flag,
-                                     tc_meta);
-            }
-            tc::fence_before_sync();
-            __syncthreads();
-            tc::fence_after_sync();
-            if (warp == kTcMmaWarp) tc::dealloc<kTcTmemCols>(tmem_base);
+        tc::fence_after_sync();
+        if constexpr (kPairs) {
+            if (tc_pairs)
+                prefix_cta_tc_pair<D>(&maps, a, smem, bars, tmem_base, warp, lane, &abort_flag, tc_meta);
+            else
+                prefix_cta_tc<D, KV>(&maps, a, smem, bars, tmem_base, warp, lane, &abort_flag, tc_meta);
         } else {
-            prefix_cta<D, KV>(&maps.k, &maps.v, a, smem, ring, bars, warp, lane, &abort_flag,
-                              id_slots);
+            prefix_cta_tc<D, KV>(&maps, a, smem, bars, tmem_base, warp, lane, &abort_flag, tc_meta);
         }
+        tc::fence_before_sync();
+        __syncthreads();
+        tc::fence_after_sync();
+        if (warp == kTcMmaWarp) tc::dealloc<kTcTmemCols>(tmem_base);
         // the prefix queue is empty: this CTA joins the suffix queue with the
         // same shared memory (every copy it issued has landed), unless every
         // suffix position is already claimed (the counter only grows, so a

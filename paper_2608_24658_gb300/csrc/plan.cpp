@@ -105,26 +105,22 @@ constexpr int64_t kFp32Slots = 3, kFp32Waves = 3;
 // (an item that grows further makes the launch's tail: build a new plan)
 constexpr int32_t kAppendSlackMin = 4, kAppendSlackMax = 64;
 constexpr int kPatchesPerTail = 6;      // words one append may change per tail item
-constexpr double kWideGroupPageCost = 1.0;   // one 16-row group of one page, in suffix pages
 constexpr double kTcPageCost = 2.0;          // one page of a tcgen05 prefix tile (tuned)
 constexpr double kTcPageCostE4m3 = 3.6;      // the same with e4m3 KV, whose suffix pages
                                              // take half the time (tuned)
+constexpr double kTcPageCostD64 = 2.5;       // the same at head_dim 64 (tuned: 16 requests x 16
+                                             // branches 201.1, 196.5, 196.5 us at 2.0, 2.5, 3.0;
+                                             // two-level 46.6, 46.6, 47.2)
 constexpr int64_t kDefaultWaitNs = 2000000000LL;
 constexpr size_t kAlign = 256;
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Time of one page of a prefix-pass tile relative to one page of the suffix
-// pass on the same SM.  The suffix pass runs 8 pages at once (one per warp);
-// a prefix tile runs one 16-row MMA group of the page per warp, so a page of
-// a tile with G groups costs G suffix pages of warp time.
-//
-// The prefix tile at head_dim 128 runs on tcgen05: one 128-row MMA per 64
-// tokens, whatever the rows, at a cost measured against the suffix pass.
-double wide_page_cost(int32_t rows, bool tensor_core_tile, bool e4m3) {
-    if (tensor_core_tile) return e4m3 ? kTcPageCostE4m3 : kTcPageCost;
-    const double groups = (rows + 15) / 16;
-    return std::max(1.0, groups * kWideGroupPageCost);
+// Time of one page of a prefix-pass tile (one 128-row MMA per 64 tokens,
+// whatever the rows) relative to one page of the suffix pass on the same SM,
+// measured.
+double wide_page_cost(int32_t head_dim, bool e4m3) {
+    return e4m3 ? kTcPageCostE4m3 : head_dim == 64 ? kTcPageCostD64 : kTcPageCost;
 }
 
 // Pieces of a run of `pages` pages under the piece length `chunk`: equal
@@ -542,7 +538,7 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
                             run.span = si;
                             run.leaf_lo = qbase[c];
                             run.wide = true;
-                            run.cost_per_page = wide_page_cost(run.nrows, true, false);
+                            run.cost_per_page = wide_page_cost(cfg->head_dim, false);
                             wide_cost += run.cost_per_page * static_cast<double>(run.pages);
                             runs.push_back(run);
                         }
@@ -569,7 +565,7 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
                                                : run.node_pages;
                         run.leaf_lo = qbase[c];
                         run.wide = true;
-                        run.cost_per_page = wide_page_cost(run.nrows, true, mode == PARASON_FP8_E4M3_KV);
+                        run.cost_per_page = wide_page_cost(cfg->head_dim, mode == PARASON_FP8_E4M3_KV);
                         wide_cost += run.cost_per_page * static_cast<double>(run.pages);
                         runs.push_back(run);
                     }
@@ -605,9 +601,7 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
                 run.leaf_lo = lo[n];
                 run.wide = wide;
                 run.cost_per_page =
-                    // bf16 and e4m3 KV at head_dim 128 run the prefix on tcgen05
-                    wide ? wide_page_cost(run.nrows, cfg->head_dim == 128, mode == PARASON_FP8_E4M3_KV)
-                         : 1.0;
+                    wide ? wide_page_cost(cfg->head_dim, mode == PARASON_FP8_E4M3_KV) : 1.0;
                 if (wide)
                     wide_cost += run.cost_per_page * static_cast<double>(P);
                 else
@@ -685,23 +679,42 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
         std::max<int64_t>(kWideBlockPages,
                           wide_units / std::max<int64_t>(1, static_cast<int64_t>(n_wide) * kWidePiecesPerCta)));
     if (!prefill && mode != PARASON_FP32 && n_wide > 0 && n_narrow_ctas > 0) {
-        int64_t entries = 0;
-        for (size_t i = 0; i < runs.size();) {
-            const size_t j = group_end(i);
-            if (runs[i].wide) {
-                int64_t per = 0, n = 0;
-                piece_split(runs[i].pages, wide_chunk, kWideBlockPages, per, n);
-                const int64_t tiles = static_cast<int64_t>(j - i);
-                entries += n * (p->tc_pairs ? (tiles + 1) / 2 : tiles);
+        auto entries_at = [&](int64_t chunk) {
+            int64_t e = 0;
+            for (size_t i = 0; i < runs.size();) {
+                const size_t j = group_end(i);
+                if (runs[i].wide) {
+                    int64_t per = 0, n = 0;
+                    piece_split(runs[i].pages, chunk, kWideBlockPages, per, n);
+                    const int64_t tiles = static_cast<int64_t>(j - i);
+                    e += n * (p->tc_pairs ? (tiles + 1) / 2 : tiles);
+                }
+                i = j;
             }
-            i = j;
-        }
+            return e;
+        };
+        const int64_t entries = entries_at(wide_chunk);
         const int32_t S = p->num_sms;
         const bool one_each =
             entries * kSpareEntriesDen <= static_cast<int64_t>(n_wide) * kSpareEntriesNum;
         if (entries > n_wide && one_each && entries <= S / 2) {
             n_wide = static_cast<int32_t>(entries);
             n_narrow_ctas = S - n_wide;
+        } else if (entries > n_wide && one_each) {
+            // one each would take too many SMs: longer pieces, at most as
+            // many as CTAs (16k prefix and 64 branches at head_dim 64: 96
+            // entries on 75 CTAs 109.7 us, 64 on 64 87.8 us; 8k and 64 branches
+            // with e4m3 KV 84.7 -> 71.4 us)
+            int64_t chunk = wide_chunk, e = entries;
+            while (e > n_wide && chunk < kMaxTileItemPages) {
+                chunk = std::min<int64_t>(kMaxTileItemPages, chunk + kWideBlockPages);
+                e = entries_at(chunk);
+            }
+            if (e <= n_wide) {
+                wide_chunk = chunk;
+                n_wide = static_cast<int32_t>(e);
+                n_narrow_ctas = S - n_wide;
+            }
         } else if (entries > n_wide && !one_each && entries <= 2 * static_cast<int64_t>(n_wide)) {
             n_wide = static_cast<int32_t>((entries + 1) / 2);
             n_narrow_ctas = S - n_wide;
