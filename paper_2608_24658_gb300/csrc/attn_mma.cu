@@ -708,6 +708,8 @@ __device__ void suffix_warp(const KvMaps &maps, const AttnArgs &a, uint32_t ring
                             int warp, int lane, WorkItem *grab) {
     using S = Shape<D, KV>;
     constexpr int NS = S::kWarpStages;
+    // pages of an item under one softmax update of the transposed step
+    constexpr int kStepPages = D == 64 ? 2 : KV::kStepPages;
     const uint32_t my_ring = ring + warp * S::kWarpRingBytes;
     const uint32_t my_bar = bars + warp * NS * 8;
     const bool skip_first = (a.debug_flags & PARASON_DEBUG_SKIP_FIRST_LOAD) && warp == 0 &&
@@ -795,19 +797,21 @@ __device__ void suffix_warp(const KvMaps &maps, const AttnArgs &a, uint32_t ring
         __syncwarp();
         const WorkItem it = grab[k % kGrabSlots];
         const float2 scl = item_scales<KV>(a, it);
-        if (it.nrows > 4 && it.nrows <= 8) {
-            // one branch of 5 to 8 q heads: the transposed step (tiles of up
-            // to 4 rows measured faster, at the tail, with the 16-row step)
+        if ((it.nrows > 4 || D == 64) && it.nrows <= 8) {
+            // one branch of 5 to 8 q heads: the transposed step (at head_dim 128
+            // tiles of up to 4 rows measured faster, at the tail, with the
+            // 16-row step; at head_dim 64, with two pages per update, slower:
+            // 16-branch step 23.3 -> 22.3 us)
             uint32_t qb[D / 16][2];
             load_q_fragments_t<D, KV>(a, it, lane, qb);
             WarpStateT<D> st;
             reset<D>(st);
             for (int pg = 0; pg < it.num_pages;) {
                 // kStepPages pages per softmax update while the item has them
-                const int np = it.num_pages - pg >= KV::kStepPages ? KV::kStepPages : 1;
-                uint32_t kb[KV::kStepPages], vb[KV::kStepPages];
+                const int np = it.num_pages - pg >= kStepPages ? kStepPages : 1;
+                uint32_t kb[kStepPages], vb[kStepPages];
 #pragma unroll
-                for (int p = 0; p < KV::kStepPages; ++p) {
+                for (int p = 0; p < kStepPages; ++p) {
                     const int c = consumed + (p < np ? p : 0);
                     const int s = c % NS;
                     kb[p] = my_ring + s * S::kStageBytes;
@@ -818,8 +822,8 @@ __device__ void suffix_warp(const KvMaps &maps, const AttnArgs &a, uint32_t ring
                 }
                 if (!ok) break;
                 const int valid = pg + np == it.num_pages ? it.last_valid : kPageSize;
-                if (KV::kStepPages > 1 && np == KV::kStepPages)
-                    pages_step_t<D, KV, KV::kStepPages>(kb, vb, valid, qb, st, scl.x, lane);
+                if (kStepPages > 1 && np == kStepPages)
+                    pages_step_t<D, KV, kStepPages>(kb, vb, valid, qb, st, scl.x, lane);
                 else
                     pages_step_t<D, KV, 1>(kb, vb, valid, qb, st, scl.x, lane);
                 __syncwarp();
