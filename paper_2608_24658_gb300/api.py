@@ -28,6 +28,19 @@ def _stream_handle(stream) -> ctypes.c_void_p:
     return ctypes.c_void_p(int(stream))
 
 
+# The current stream's handle without a Stream object for it (about a fifth of
+# a small step's host time).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream_int(stream) -> int:
+    if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
+        stream = torch.cuda.current_stream()
+    return stream.cuda_stream if isinstance(stream, torch.cuda.Stream) else int(stream)
+
+
 def _i32(a) -> np.ndarray:
     return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
 
@@ -193,39 +206,48 @@ class Plan:
         """One decode step; returns (out, lse).  Asynchronous on ``stream``.
         ``q``, ``out`` and ``lse`` may be pinned host tensors: the kernels
         then read q from, and write the result to, host memory directly."""
+        # (small steps wait for this code: tensors are looked at once, and
+        # pointers go to the library as integers)
         L, Hq, Hkv, d = self.num_leaves, self.num_q_heads, self.num_kv_heads, self.head_dim
         qd, kvd = _Q_DTYPES[self.mode], _KV_DTYPES[self.mode]
-        if (q.dtype != qd or tuple(q.shape) != (L, Hq, d) or not q.is_contiguous()
-                or not (q.is_cuda or q.is_pinned())):
+        q_cuda = q.is_cuda
+        if (q.dtype != qd or q.shape != (L, Hq, d) or not q.is_contiguous()
+                or not (q_cuda or q.is_pinned())):
             raise ValueError(f"q must be a contiguous cuda (or pinned host) {qd} tensor of "
                              f"shape {(L, Hq, d)}")
         dev = k_pages.device
         for name, t in (("k_pages", k_pages), ("v_pages", v_pages)):
-            if (t.dtype != kvd or t.dim() != 4 or tuple(t.shape[1:]) != (Hkv, 16, d)
-                    or t.shape[0] < self.num_physical_pages or not t.is_contiguous()
-                    or not t.is_cuda or t.device != dev):
+            shape = t.shape
+            if (t.dtype != kvd or shape[1:] != (Hkv, 16, d) or shape[0] < self.num_physical_pages
+                    or not t.is_contiguous() or not t.is_cuda or t.device != dev):
                 raise ValueError(f"{name} must be a contiguous cuda {kvd} tensor "
                                  f"[>= {self.num_physical_pages}, {Hkv}, 16, {d}] on one device")
-        if q.is_cuda and q.device != dev:
+        if q_cuda and q.device != dev:
             raise ValueError(f"q must be on {dev}")
         if out is None:
-            out = torch.empty_like(q) if q.is_cuda else torch.empty(q.shape, dtype=q.dtype).pin_memory()
+            out = torch.empty_like(q) if q_cuda else torch.empty(q.shape, dtype=q.dtype).pin_memory()
         if lse is None and want_lse:
-            lse = (torch.empty((L, Hq), dtype=torch.float32, device=dev) if q.is_cuda else
+            lse = (torch.empty((L, Hq), dtype=torch.float32, device=dev) if q_cuda else
                    torch.empty((L, Hq), dtype=torch.float32).pin_memory())
         if workspace is None:
             workspace = self.workspace(dev)
+        ks = vs = None
         if self.mode == "fp8":
             if k_scale is None or v_scale is None:
                 raise ValueError("fp8 mode needs k_scale and v_scale")
             for s in (k_scale, v_scale):
                 if s.dtype != torch.float32 or s.numel() != Hkv or not s.is_cuda:
                     raise ValueError(f"scales must be cuda float32 [{Hkv}]")
+        if k_scale is not None:
+            ks = k_scale.data_ptr()
+        if v_scale is not None:
+            vs = v_scale.data_ptr()
         st = _lib.load().parason_attn_decode(
-            self.handle, _ptr(q), _ptr(k_pages), _ptr(v_pages), _ptr(k_scale), _ptr(v_scale),
-            _ptr(out), _ptr(lse), _ptr(workspace), workspace.numel() * workspace.element_size(),
-            _stream_handle(stream))
-        check(st, "parason_attn_decode")
+            self.handle, q.data_ptr(), k_pages.data_ptr(), v_pages.data_ptr(), ks, vs,
+            out.data_ptr(), None if lse is None else lse.data_ptr(), workspace.data_ptr(),
+            workspace.numel() * workspace.element_size(), _stream_int(stream))
+        if st:
+            check(st, "parason_attn_decode")
         return out, lse
 
     def decode_no_alloc(self, q: torch.Tensor, k_pages: torch.Tensor, v_pages: torch.Tensor,
@@ -332,10 +354,11 @@ def lse_merge(o_a: torch.Tensor, lse_a: torch.Tensor, o_b: torch.Tensor, lse_b: 
     o_out = torch.empty_like(o_a) if o_out is None else o_out
     lse_out = torch.empty_like(lse_a) if lse_out is None else lse_out
     mode = _lib.MODES["fp32" if o_a.dtype == torch.float32 else "bf16"]
-    st = _lib.load().parason_lse_merge(_ptr(o_a), _ptr(lse_a), _ptr(o_b), _ptr(lse_b),
-                                       _ptr(o_out), _ptr(lse_out), rows, d, mode,
-                                       _stream_handle(stream))
-    check(st, "parason_lse_merge")
+    st = _lib.load().parason_lse_merge(o_a.data_ptr(), lse_a.data_ptr(), o_b.data_ptr(),
+                                       lse_b.data_ptr(), o_out.data_ptr(), lse_out.data_ptr(),
+                                       rows, d, mode, _stream_int(stream))
+    if st:
+        check(st, "parason_lse_merge")
     return o_out, lse_out
 
 
