@@ -73,7 +73,10 @@ constexpr int kPrefillBlockPages = parason::kPrefillBoxPages;   // a prefill til
 // kMinPiecePages and at most kMaxPiecePages pages).  Same-box A/B against
 // 3: two-level step 79.7 -> 78.8 us, the Llama-3 shape level (its pieces
 // were at an 8-page floor); 2 made the Llama-3-shape step 2 us slower.
-constexpr double kNarrowPiecesPerWarp = 2.5;
+// With e4m3 KV 2: two-level 64.5 -> 62.5 us, 8k prefix and 64 branches 71.0 ->
+// 68.3 (with bf16 KV slower: 16 branches 31.6 -> 33.0 us, and at head_dim 64
+// 16 x 16 branches 195 -> 205).
+constexpr double kNarrowPiecesPerWarp = 2.5, kNarrowPiecesPerWarpE4m3 = 2.0;
 constexpr double kWideProvision = 1.15;   // prefix CTAs relative to the cost model
 // Decode: up to this many prefix queue entries per prefix CTA (num / den)
 // become one CTA each; up to two, two entries each
@@ -823,11 +826,12 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
             if (!cut(r, chunk, 1)) return PARASON_EUNSUPPORTED;
     } else {
         const int64_t total_warps = static_cast<int64_t>(p->num_sms) * p->suffix_warps;
+        const double pieces = mode == PARASON_FP8_E4M3_KV ? kNarrowPiecesPerWarpE4m3 : kNarrowPiecesPerWarp;
         const int64_t narrow_chunk = std::min<int64_t>(
             kMaxPiecePages,
             std::max<int64_t>(kMinPiecePages,
                               static_cast<int64_t>(static_cast<double>(narrow_pages) /
-                                                   (kNarrowPiecesPerWarp * std::max<int64_t>(1, total_warps)))));
+                                                   (pieces * std::max<int64_t>(1, total_warps)))));
         p->narrow_chunk = narrow_chunk;
         if (prefill && n_wide > 0 && !runs.empty()) {
             std::vector<PrefillGroup> groups;
