@@ -131,7 +131,10 @@ cudaError_t attn_mma_ctas_per_sm(int head_dim, int mode, int *ctas_per_sm);
 // blocks whose pages are consecutive in the pool.  k_box / v_box: one box is
 // kBoxPages pages of one kv head that are consecutive in the pool, its column
 // blocks one after another (the layout the per-block boxes of k / v give):
-// one page in a decode plan, a 128-token block in a prefill plan.
+// one page in a decode plan, a 128-token block in an e4m3 prefill plan.  A
+// prefill plan with bf16 KV has k and v alone, and they are whole pages: k as
+// [8-row half][column block][8 rows], so that pages staged one after another
+// have their 8-row groups 2 KB apart, v as the decode plan's page box.
 constexpr int kTcRunPages = 4;
 constexpr int kDecodeBoxPages = 1, kPrefillBoxPages = 8;
 struct KvMaps {

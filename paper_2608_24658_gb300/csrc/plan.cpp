@@ -1222,6 +1222,22 @@ parason_status encode_kv_box_map(CUtensorMap *map, const void *pages, int64_t nu
     return r == CUDA_SUCCESS ? PARASON_OK : PARASON_ECUDA;
 }
 
+// A page of one kv head (head_dim 128, bf16) as [8-row half][column block][8
+// rows of 128 bytes]: dim0 = 128 bytes of a segment, dim1 = row of a half
+// (stride one token row), dim2 = segment, dim3 = half, dim4 = (page * H_kv +
+// kv_head).
+parason_status encode_kv_half_map(CUtensorMap *map, const void *pages, int64_t num_phys, int32_t H_kv) {
+    auto fn = encode_fn();
+    if (!fn) return PARASON_ECUDA;
+    const cuuint64_t dims[5] = {64, 8, 2, 2, static_cast<cuuint64_t>(num_phys) * H_kv};
+    const cuuint64_t strides[4] = {256, 128, 2048, 4096};
+    const cuuint32_t box[5] = {64, 8, 2, 2, 1}, estr[5] = {1, 1, 1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(pages), dims, strides, box,
+                    estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? PARASON_OK : PARASON_ECUDA;
+}
+
 parason_status record_event(parason_plan_s *p, int which, cudaStream_t stream) {
     if (p->timing_cap <= 0 || p->timing_n >= p->timing_cap) return PARASON_OK;
     cudaEvent_t ev = p->events[3 * p->timing_n + which];
@@ -1573,12 +1589,14 @@ parason_status parason_attn_decode(parason_plan p, const void *q, const void *k_
             {
                 std::lock_guard<std::mutex> lock(p->tm_mutex);
                 const int32_t H = p->cfg.num_kv_heads, mode = p->cfg.mode;
+                const bool halves = p->prefill && mode == PARASON_BF16;
                 if (p->tm_k_ptr != k_pages) {
                     p->tm_k_ptr = nullptr;
-                    st = encode_kv_map(&p->tm.k, k_pages, p->num_phys, H, d, mode);
-                    if (st == PARASON_OK)
+                    st = halves ? encode_kv_half_map(&p->tm.k, k_pages, p->num_phys, H)
+                                : encode_kv_map(&p->tm.k, k_pages, p->num_phys, H, d, mode);
+                    if (st == PARASON_OK && !halves)
                         st = encode_kv_run_map(&p->tm.k_run, k_pages, p->num_phys, H, d, mode);
-                    if (st == PARASON_OK)
+                    if (st == PARASON_OK && !halves)
                         st = encode_kv_box_map(&p->tm.k_box, k_pages, p->num_phys, H, d, mode,
                                                p->prefill);
                     if (st != PARASON_OK) return st;
@@ -1586,10 +1604,11 @@ parason_status parason_attn_decode(parason_plan p, const void *q, const void *k_
                 }
                 if (p->tm_v_ptr != v_pages) {
                     p->tm_v_ptr = nullptr;
-                    st = encode_kv_map(&p->tm.v, v_pages, p->num_phys, H, d, mode);
-                    if (st == PARASON_OK)
+                    st = halves ? encode_kv_box_map(&p->tm.v, v_pages, p->num_phys, H, d, mode, false)
+                                : encode_kv_map(&p->tm.v, v_pages, p->num_phys, H, d, mode);
+                    if (st == PARASON_OK && !halves)
                         st = encode_kv_run_map(&p->tm.v_run, v_pages, p->num_phys, H, d, mode);
-                    if (st == PARASON_OK)
+                    if (st == PARASON_OK && !halves)
                         st = encode_kv_box_map(&p->tm.v_box, v_pages, p->num_phys, H, d, mode,
                                                p->prefill);
                     if (st != PARASON_OK) return st;

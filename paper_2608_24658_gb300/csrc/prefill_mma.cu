@@ -12,10 +12,13 @@
 //   warps 0-3   tile A: softmax (thread r owns row r, TMEM lane r), the next
 //               pair's Q rows, then the row's (m, l) and O
 //   warps 4-7   tile B: the same
-//   warp 8      producer: TMA of K, then V, of each block into a ring; one
-//               32 KB box (16 KB in e4m3) when the block's 8 pages are
-//               consecutive in the pool, else a box per 4 pages and column
-//               block, or per page and column block
+//   warp 8      producer: TMA of K, then V, of each block into a ring.  bf16:
+//               a 4 KB box per page, one lane each, laid out so that the MMA
+//               reads 8 pages anywhere in the pool as one operand (a 2 KB box
+//               per page and column block took permuted pages from 495 to 595
+//               us on the join; one 32 KB box for consecutive pages is level).
+//               e4m3: one 16 KB box when the block's 8 pages are consecutive,
+//               else a box per 4 pages or per page
 //   warp 9      MMA issuer: S_t = Q_t K^T (M 128, N 128, both operands in
 //               shared memory) and O_t += P_t V (P in TMEM) for t = A, B in
 //               turn (two issuers let the tiles fall into step, both in their
@@ -74,6 +77,7 @@ constexpr int kBlockPages = kPrefillBoxPages;                  // 8
 constexpr int kBlockTokens = kBlockPages * kPageSize;          // 128
 constexpr int kColBlockBytes = kBlockTokens * 128;             // 16 KB: 128 keys x 128 bytes
 constexpr int kSlotBytes = 2 * kColBlockBytes;                 // 32 KB: K or V of a block, 16-bit
+constexpr int kPagedBytes = kSlotBytes / kBlockPages;          // 4 KB: a page of it
 constexpr int kRawSlotBytes = kBlockTokens * 128;              // 16 KB: the same in e4m3
 constexpr int kQColBlockBytes = kRows * 128;                   // 16 KB
 constexpr int kQBytes = 2 * kQColBlockBytes;                   // 32 KB a tile
@@ -227,8 +231,8 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
         progress = 0;
         for (int i = 0; i < kBars; ++i) dev::mbar_init(bar(i), bar_count(i, F8));
         dev::fence_mbar_init();
-        dev::prefetch_tensormap(&maps.k_box);
-        dev::prefetch_tensormap(&maps.v_box);
+        dev::prefetch_tensormap(F8 ? &maps.k_box : &maps.k);
+        dev::prefetch_tensormap(F8 ? &maps.v_box : &maps.v);
     }
     if (warp == kMmaWarp) tc::alloc<kTmemCols>(dev::smem_addr(&tmem_base));
     tc::fence_before_sync();
@@ -460,12 +464,14 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                                 ok = false;
                                 break;
                             }
-                            const uint32_t vst = ring + vs * kSlotBytes + h * kHalfTokens * 128;
+                            const uint32_t vst = ring + vs * kSlotBytes;
                             const int n16 = (kHalfTokens - valid[h]) * 2 * 8;
                             for (int q = r; q < n16; q += kRows) {
-                                const int row = valid[h] + q / 16, cb = (q / 8) & 1, c = q & 7;
+                                const int row = h * kHalfTokens + valid[h] + q / 16, cb = (q / 8) & 1;
+                                const uint32_t at = row / kPageSize * kPagedBytes + cb * (kPagedBytes / 2) +
+                                                    row % kPageSize * 128;
                                 asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(
-                                                 vst + cb * kColBlockBytes + row * 128 + (c << 4)),
+                                                 vst + at + ((q & 7) << 4)),
                                              "r"(0u)
                                              : "memory");
                             }
@@ -668,11 +674,6 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
             const bool skip_first = a.debug_flags & PARASON_DEBUG_SKIP_FIRST_LOAD;
             const int page_rows = a.num_kv_heads * kPageSize;   // TMA rows between consecutive pages
             const uint64_t pol = dev::l2_evict_normal_policy();
-            // this lane's part of a slot that is not one run of pages: page j of
-            // half h, column block cb (16-bit elements: 16 lanes; e4m3: 8)
-            const int h = F8 ? lane >> 2 : lane >> 3, j = F8 ? lane & 3 : (lane >> 1) & 3;
-            const int cb = F8 ? 0 : lane & 1;
-            const bool mine = lane < (F8 ? 8 : 16);
             int last_issue[NS];
             for (int s = 0; s < NS; ++s) last_issue[s] = -1;
             int pos = 0, blk = 0, st = 0;                // slot st = pos % NS
@@ -723,8 +724,7 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                         valid[hh] = max(0, min(valid[hh], tokens - (i * kBlockTokens + hh * kHalfTokens)));
                     }
                     if (lane == 0) valid_ring[blk % kValidRing] = valid[0] | (valid[1] << 8);
-                    const uint32_t f8 = (follows >> w0) & 0xffu;
-                    const bool whole = ((pool >> w0) & 1u) && (f8 & 0xfeu) == 0xfeu;
+                    const bool whole = F8 && ((pool >> w0) & 1u) && ((follows >> w0) & 0xfeu) == 0xfeu;
                     const int32_t row0 = __shfl_sync(0xffffffffu, win, w0) & ~(kPageSize - 1);
                     for (int op = 0; op < 2; ++op, ++pos, st = st + 1 == NS ? 0 : st + 1) {
                         if (pos >= NS && !tc_warp_wait(bar(kEmptyBar + st), ((pos / NS) - 1) & 1, limit, abort,
@@ -744,17 +744,32 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                             continue;
                         }
                         __syncwarp();
-                        const uint32_t dst = dst0 + cb * kColBlockBytes + h * kHalfTokens * 128;
+                        if constexpr (!F8) {
+                            // a box of 4 KB per page (lane: page): K as [half][column
+                            // block][8 rows], V as [column block][16 rows]
+                            const int32_t pr = __shfl_sync(0xffffffffu, win, w0 + (lane & 7));
+                            const uint32_t dst = dst0 + (lane & 7) * kPagedBytes;
+                            if (lane < kBlockPages) {
+                                if (op == 0)
+                                    dev::tma_load_5d_hint(dst, &maps.k, 0, 0, 0, 0, pr / kPageSize, fb, pol);
+                                else
+                                    dev::tma_load_4d_hint(dst, &maps.v, 0, 0, 0, pr / kPageSize, fb, pol);
+                            }
+                            continue;
+                        }
+                        // e4m3: a box per run of 4 pages, or per page (lane: page j of half h)
+                        const int h = lane >> 2, j = lane & 3;
+                        const uint32_t dst = dst0 + h * kHalfTokens * 128;
                         const int lane_pg = w0 + ((4 * h + j) & 7);
                         const int32_t my_row = __shfl_sync(0xffffffffu, win, lane_pg) & ~(kPageSize - 1);
                         const int first = w0 + 4 * (h & 1);
                         const bool my_run = ((pool >> first) & 1u) && ((follows >> first) & 0xeu) == 0xeu;
-                        if (mine && my_run) {
+                        if (lane < kBlockPages && my_run) {
                             if (j == 0)
-                                dev::tma_load_5d_hint(dst, op ? &maps.v_run : &maps.k_run, 0, cb, 0, kvh,
+                                dev::tma_load_5d_hint(dst, op ? &maps.v_run : &maps.k_run, 0, 0, 0, kvh,
                                                       my_row / page_rows, fb, pol);
-                        } else if (mine) {
-                            dev::tma_load_3d(dst + j * kPageSize * 128, op ? &maps.v : &maps.k, 0, cb,
+                        } else if (lane < kBlockPages) {
+                            dev::tma_load_3d(dst + j * kPageSize * 128, op ? &maps.v : &maps.k, 0, 0,
                                              my_row, fb);
                         }
                     }
@@ -775,7 +790,6 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                                          : tc::idesc_bf16_f32(kRows, kBlockTokens, false);
             constexpr uint32_t kIdPV = F8 ? tc::idesc_f16_f32(kRows, kDim, true)
                                           : tc::idesc_bf16_f32(kRows, kDim, true);
-            static_assert(kColBlockBytes == kQColBlockBytes, "one offset for Q and K");
             // A wait that runs out leaves its mark, and the warp goes on together
             // to the next point where it looks (lanes that part would leave the
             // others waiting in elect.sync; what is issued in between works on
@@ -788,8 +802,14 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                 }
             };
             auto failed = [&]() { return __any_sync(0xffffffffu, bad) != 0; };
-            const uint64_t desc_k = tc::smem_desc_sw128(ring, 16, 1024);
-            const uint64_t desc_v = tc::smem_desc_sw128(ring, kColBlockBytes, 1024);
+            // K and V of a block: with bf16 KV page by page (8-row groups of K 2
+            // KB apart, column blocks 1 KB; of V a 16-token step 4 KB, column
+            // blocks 2 KB), widened e4m3 as column blocks of 128 tokens
+            constexpr uint32_t kKGroup = F8 ? 1024 : 2048, kKCol = F8 ? kColBlockBytes : 1024;
+            constexpr uint32_t kVStep = F8 ? kPageSize * 128 : kPagedBytes;
+            constexpr uint32_t kVCol = F8 ? kColBlockBytes : kPagedBytes / 2;
+            const uint64_t desc_k = tc::smem_desc_sw128(ring, 16, kKGroup);
+            const uint64_t desc_v = tc::smem_desc_sw128(ring, kVCol, 1024);
             const uint64_t desc_q = tc::smem_desc_sw128(q_smem, 16, 1024);
             int st = 0, ph = 0;              // ring slot of the next operand, and its phase
             auto advance = [&]() {
@@ -806,8 +826,9 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                 if (tc::elect_one()) {
 #pragma unroll
                     for (int ks = 0; ks < kDim / 16; ++ks) {
-                        const uint32_t off = ((ks >> 2) * kColBlockBytes + (ks & 3) * 32) >> 4;
-                        tc::mma_bf16(tS, qd + off, kd + off, kIdS, ks > 0);
+                        const uint32_t off = ((ks >> 2) * kQColBlockBytes + (ks & 3) * 32) >> 4;
+                        const uint32_t koff = ((ks >> 2) * kKCol + (ks & 3) * 32) >> 4;
+                        tc::mma_bf16(tS, qd + off, kd + koff, kIdS, ks > 0);
                     }
                     // the commit completes with the product; the plain arrive
                     // carries the producer's writes (valid_ring) along
@@ -852,8 +873,7 @@ __global__ void __launch_bounds__(Cfg<F8>::kThreads, 1)
                             if (tc::elect_one()) {
 #pragma unroll
                                 for (int kk = 4 * hf; kk < 4 * hf + 4; ++kk)
-                                    tc::mma_bf16_tmem_a(tO, tP + 8u * kk,
-                                                        vd + static_cast<uint32_t>((kk * 2048) >> 4), kIdPV,
+                                    tc::mma_bf16_tmem_a(tO, tP + 8u * kk, vd + ((kk * kVStep) >> 4), kIdPV,
                                                         i > 0 || kk > 0);
                                 if (hf == 1 && t == last) tc::commit(bar(kEmpty + sv));
                                 if (hf == 1 && i == nb - 1) tc::commit(bar(kOFull + t));

@@ -13,11 +13,13 @@ namespace tc {
 // along the 8-row direction, `lbo` the distance between atoms along the
 // other direction (used by MN-major operands, ignored by K-major ones whose
 // 16-element K step stays inside one 128-byte row).
+__host__ __device__ constexpr uint64_t smem_desc_stride(uint32_t lbo, uint32_t sbo) {
+    return (static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16) | (static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32);
+}
+
 __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t smem_addr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = 0;
+    uint64_t d = smem_desc_stride(lbo, sbo);
     d |= static_cast<uint64_t>((smem_addr >> 4) & 0x3FFFu);
-    d |= static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16;
-    d |= static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32;
     d |= static_cast<uint64_t>(1) << 46;       // descriptor version for sm_100 family
     d |= static_cast<uint64_t>(2) << 61;       // 128-byte swizzle
     return d;
