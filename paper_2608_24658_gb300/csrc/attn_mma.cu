@@ -898,7 +898,9 @@ __device__ void suffix_warp(const KvMaps &maps, const AttnArgs &a, uint32_t ring
 //   warps 4-7   epilogue: once an item's O is complete, stores its rows to the
 //               partials and loads the Q rows of the item two ahead into the
 //               TMEM Q buffer that item frees (Q of items 0 and 1 at start);
-//               with e4m3 KV they also convert every staged block to f16
+//               with e4m3 KV they also convert every staged block to f16, and
+//               an item's Q is filled before its first block, since the next
+//               item is known only when this one nears its end (kTcWantBlocks)
 //
 // At head_dim 64 a stage is 16 KB and every product half as deep or as wide
 // (against a prefix pass on mma.sync, 8 warps of 16 rows page by page: 4 requests
@@ -927,8 +929,15 @@ constexpr int kTcF8Bytes = kTcBlockTokens * 128;              // 8 KB: K (or V) 
 constexpr int kTcF8StageBytes = 2 * kTcF8Bytes;
 constexpr int kTcF8Stages = 4;                                 // raw e4m3 stages
 constexpr int kTcCvStages = 4;
+// The scheduler of an e4m3 tile pulls the next item when the producer has this
+// many blocks of the present one left (4 to 12 measured the same), not as soon
+// as a metadata slot is free: with the pull up to four items ahead, CTAs held
+// entries that others had time for (a 16k prefix over 128 branches 218 ->
+// 193 us, a two-level tree 62.5 -> 60.1 us).  bf16 tiles stream without the
+// conversion, and measured level (head_dim 128) or 1% slower (64) this way.
+constexpr int kTcWantBlocks = 8;
 constexpr int kTcCvOffset = kTcF8Stages * kTcF8StageBytes;    // 64 KB
-static_assert(kTcF8Stages <= kTcStages, "raw e4m3 stages use the ring's barriers");
+static_assert(kTcF8Stages < kTcStages, "raw e4m3 stages and kBarWant use the ring's barriers");
 static_assert(kTcCvOffset + kTcCvStages * kTcStageBytes <= kTcRingBytes, "e4m3 rings fit");
 constexpr int kTcTmemCols = 512;
 constexpr uint32_t kTmemO = 0, kTmemS = 256, kTmemQ = 384;    // TMEM column bases
@@ -979,7 +988,10 @@ enum TcBar : int {
     kBarDrain = kBarMetaEmpty + kTcMeta,     // both issuers' commits -> issuers, before TMEM is freed
     kBarCvFull,                              // [kTcCvStages] converters (4 arrivals) -> MMA
     kBarCvEmpty = kBarCvFull + kTcCvStages,  // [kTcCvStages] MMA commit -> converters
-    kTcBars = kBarCvEmpty + kTcCvStages
+    kTcBars = kBarCvEmpty + kTcCvStages,
+    // producer -> scheduler: pull the next item (e4m3 tiles, which use
+    // kTcF8Stages of the kTcStages staging barriers)
+    kBarWant = kBarKvFull + kTcF8Stages
 };
 
 // arrivals each barrier waits for; with e4m3 KV the 4 converter warps free
@@ -1064,8 +1076,13 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
         // ------------------------------------------------------------ scheduler
         for (int k = 0;; ++k) {
             const int s = k % kTcMeta;
-            if (k >= kTcMeta &&
-                !tc_warp_wait(bar(kBarMetaEmpty + s), ((k / kTcMeta) - 1) & 1, limit, abort_flag, lane)) {
+            bool fine = true;
+            if constexpr (kF8) {
+                if (k > 0) fine = tc_warp_wait(bar(kBarWant), (k - 1) & 1, limit, abort_flag, lane);
+            }
+            if (!fine ||
+                (k >= kTcMeta && !tc_warp_wait(bar(kBarMetaEmpty + s), ((k / kTcMeta) - 1) & 1, limit,
+                                               abort_flag, lane))) {
                 if (lane == 0) tc_fail(a, abort_flag, kSiteProducerEmpty);
                 break;
             }
@@ -1122,6 +1139,9 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
             const int np = m.it.num_pages;
             const int nb = tc_blocks(np);
             for (int bi = 0; bi < nb; ++bi, ++blk) {
+                if constexpr (kF8) {
+                    if (bi == max(0, nb - kTcWantBlocks) && lane == 0) dev::mbar_arrive(bar(kBarWant));
+                }
                 const int s = blk % NS;
                 if (blk >= NS &&
                     !tc_warp_wait(bar(kBarKvEmpty + s), ((blk / NS) - 1) & 1, limit, abort_flag,
@@ -1501,18 +1521,13 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                 if (lane == 0) dev::mbar_arrive(bar(kBarKvEmpty + s));
                 return true;
             };
-            // store item j's O; load item j + 2's Q into the buffer j frees
-            auto finish = [&](int j, bool next_exists) -> bool {
+            // store item j's O
+            auto finish = [&](int j) -> bool {
                 const WorkItem it = meta[j % kTcMeta].it;
                 if (!tc_warp_wait(bar(kBarOFull + (j & 1)), (j >> 1) & 1, limit, abort_flag, lane))
                     return false;
                 tc::fence_after_sync();
-                const bool has_j2 = next_exists && has_item(j + 2);
-                if (!ok) return false;
-                uint4 qv[D / 8];
-                if (has_j2) fetch_q(j + 2, qv);
                 store_o(j, it);
-                if (has_j2) put_q(j + 2, qv);
                 tc::fence_before_sync();
                 __syncwarp();
                 if (lane == 0) {
@@ -1521,30 +1536,22 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
                 }
                 return true;
             };
-            if (has_item(0)) {
+            bool have = has_item(0);
+            for (int k = 0, gb = 0; ok && have; ++k) {
+                // item k's Q: its buffer was freed by item k - 2, whose O is stored
                 uint4 qv[D / 8];
-                fetch_q(0, qv);
-                put_q(0, qv);
-                if (has_item(1)) {
-                    fetch_q(1, qv);
-                    put_q(1, qv);
+                fetch_q(k, qv);
+                put_q(k, qv);
+                const WorkItem it = meta[k % kTcMeta].it;
+                const int nb = tc_blocks(it.num_pages);
+                const int tokens = (it.num_pages - 1) * kPageSize + it.last_valid;
+                for (int i = 0; i < nb && ok; ++i, ++gb) {
+                    ok = convert(gb, min(kTcBlockTokens, tokens - i * kTcBlockTokens));
+                    if (ok && k > 0 && i == min(1, nb - 1)) ok = finish(k - 1);
                 }
-                for (int k = 0, gb = 0; ok; ++k) {
-                    const WorkItem it = meta[k % kTcMeta].it;
-                    const int nb = tc_blocks(it.num_pages);
-                    const int tokens = (it.num_pages - 1) * kPageSize + it.last_valid;
-                    for (int i = 0; i < nb && ok; ++i, ++gb) {
-                        ok = convert(gb, min(kTcBlockTokens, tokens - i * kTcBlockTokens));
-                        if (ok && k > 0 && i == min(1, nb - 1)) ok = finish(k - 1, true);
-                    }
-                    if (!ok) break;
-                    const bool more = has_item(k + 1);
-                    if (!ok) break;
-                    if (!more) {
-                        ok = finish(k, false);
-                        break;
-                    }
-                }
+                if (!ok) break;
+                have = has_item(k + 1);
+                if (ok && !have) ok = finish(k);
             }
             if (!ok && lane == 0) tc_fail(a, abort_flag, kSiteConsumerFull);
             return;

@@ -109,8 +109,13 @@ constexpr int64_t kFp32Slots = 3, kFp32Waves = 3;
 constexpr int32_t kAppendSlackMin = 4, kAppendSlackMax = 64;
 constexpr int kPatchesPerTail = 6;      // words one append may change per tail item
 constexpr double kTcPageCost = 2.0;          // one page of a tcgen05 prefix tile (tuned)
-constexpr double kTcPageCostE4m3 = 3.6;      // the same with e4m3 KV, whose suffix pages
-                                             // take half the time (tuned)
+// The same with e4m3 KV, and a tile's start in pages, which weighs there: the
+// converters fill an item's Q before its first block (tuned; per page alone, at
+// 3.6, 3.2, 2.6: a 16k prefix over 128 branches 192, 189, 184 us, 4 requests
+// of a 2k prefix over 16 branches 76.7, 76.7, 80.6; 2.6 and the start 184 and
+// 77.1; a 32k prefix over 128 branches of 4k to 16k 521, 521, 506)
+constexpr double kTcPageCostE4m3 = 2.6;
+constexpr int64_t kTcStartPagesE4m3 = 24;
 constexpr double kTcPageCostD64 = 2.5;       // the same at head_dim 64 (tuned: 16 requests x 16
                                              // branches 201.1, 196.5, 196.5 us at 2.0, 2.5, 3.0;
                                              // two-level 46.6, 46.6, 47.2)
@@ -606,7 +611,8 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
                 run.cost_per_page =
                     wide ? wide_page_cost(cfg->head_dim, mode == PARASON_FP8_E4M3_KV) : 1.0;
                 if (wide)
-                    wide_cost += run.cost_per_page * static_cast<double>(P);
+                    wide_cost += run.cost_per_page *
+                                 static_cast<double>(P + (mode == PARASON_FP8_E4M3_KV ? kTcStartPagesE4m3 : 0));
                 else
                     narrow_pages += P;
                 runs.push_back(run);
