@@ -23,7 +23,13 @@
 // What bounds it: HBM.  A page of a 4-row tile is 16 KB (d 128) for about 430
 // warp instructions.  16 branches of 512 to 4096 tokens under a 2048-token
 // prefix, 32 q / 8 kv heads, d 128 (327 MB of KV, 48 us at 6.8 TB/s): 442 us
-// with a warp reduction per (token, row) and direct global loads, 73 us now.
+// with a warp reduction per (token, row) and direct global loads, 70 us with
+// K and V of a page copied and awaited together, 65.5 us now.  A tile of at most
+// 4 rows has one stage per warp at d 128, which was empty while its copies
+// came: its K is now refilled as soon as the scores are made, its V after the
+// page (16 kv heads of one q head each: 48.4 -> 45.4 us).  Wider tiles keep one
+// copy: there the pages are shared and the FMAs bound it (two-level tree of
+// 64 q heads 75 us; 80 us with split copies).
 #include "device_common.cuh"
 #include "internal.h"
 
@@ -44,6 +50,8 @@ struct F32 {
     static constexpr int kStageBytes = 2 * kTensorBytes;
     static constexpr int kStages = kRing / kStageBytes;       // 4 (d 128) or 8 (d 64)
     static constexpr int kChunks = D / 32;                    // 16-byte chunks of a row per lane
+    // (at d 64 a warp has two stages and the split copies were 8% slower)
+    static constexpr bool kSplit = D == 128;
     static_assert(kStages % kWarps == 0, "a stage's next page belongs to the same warps");
 };
 
@@ -73,13 +81,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     extern __shared__ __align__(128) uint8_t ring_mem[];
     __shared__ float sc_o[kWarps][kWarpRows][D];
     __shared__ float2 sc_ml[kWarps][kWarpRows];
-    __shared__ __align__(8) uint64_t bars[2 * NS];
+    __shared__ __align__(8) uint64_t bars[3 * NS];
     __shared__ int failed;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int s = lane & 7, tg = lane >> 3;            // chunk and token group of the lane
     const int b0 = lane & 1, b1 = (lane >> 1) & 1, b2 = (lane >> 2) & 1;
     const uint32_t ring = dev::smem_addr(ring_mem);
-    const uint32_t full = dev::smem_addr(bars), empty = full + 8 * NS;
+    const uint32_t full = dev::smem_addr(bars), empty = full + 8 * NS, vfull = empty + 8 * NS;
 
     dev::grid_wait();
     const WorkItem it = a.items[blockIdx.x];
@@ -87,11 +95,15 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     const int RG = row_groups == 3 ? 4 : row_groups;
     const int PG = kWarps / RG;                        // warps that share a row group's pages
     const int rgi = warp / PG, pgi = warp % PG;
+    // K and V copied, awaited and refilled one by one: a stage's K comes while
+    // the page's softmax and V run
+    const bool split = S::kSplit && row_groups == 1;
     if (threadIdx.x == 0) {
         failed = 0;
         for (int i = 0; i < NS; ++i) {
             dev::mbar_init(full + 8 * i, 1);
             dev::mbar_init(empty + 8 * i, row_groups);
+            dev::mbar_init(vfull + 8 * i, 1);
         }
         dev::fence_mbar_init();
     }
@@ -101,20 +113,26 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     // page pg of the item into its stage; pages pg, pg + PG, ... are this
     // warp's, and the warps of row group 0 load them
     const int first_ids = lane < it.num_pages ? a.page_ids[it.page_pos + lane] : 0;
-    auto load = [&](int pg) {
+    auto load = [&](int pg, bool k, bool v) {
         const int page = pg < 32 ? __shfl_sync(0xffffffffu, first_ids, pg) : a.page_ids[it.page_pos + pg];
         if (lane == 0) {
             const int64_t off = (static_cast<int64_t>(page) * a.num_kv_heads + it.kv_head) * kPageSize * D;
-            const uint32_t dst = ring + (pg % NS) * S::kStageBytes, bar = full + 8 * (pg % NS);
-            dev::mbar_arrive_expect_tx(bar, S::kStageBytes);
-            bulk_load(dst, kp + off, S::kTensorBytes, bar);
-            bulk_load(dst + S::kTensorBytes, vp + off, S::kTensorBytes, bar);
+            const uint32_t dst = ring + (pg % NS) * S::kStageBytes;
+            const uint32_t bar = full + 8 * (pg % NS), vbar = split ? vfull + 8 * (pg % NS) : bar;
+            if (k) {
+                dev::mbar_arrive_expect_tx(bar, split ? S::kTensorBytes : S::kStageBytes);
+                bulk_load(dst, kp + off, S::kTensorBytes, bar);
+            }
+            if (v) {
+                if (split) dev::mbar_arrive_expect_tx(vbar, S::kTensorBytes);
+                bulk_load(dst + S::kTensorBytes, vp + off, S::kTensorBytes, vbar);
+            }
         }
     };
     const bool active = rgi < row_groups;
     int loaded = pgi, used = pgi;                      // next own page to load, to use
     if (rgi == 0)
-        for (; loaded < it.num_pages && loaded < NS; loaded += PG) load(loaded);
+        for (; loaded < it.num_pages && loaded < NS; loaded += PG) load(loaded, true, true);
 
     Pairs q[kWarpRows][NC], o[kWarpRows][NC];
 #pragma unroll
@@ -136,7 +154,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     // this lane's scores: rows 2 b0 and 2 b0 + 1 of token 4 (2 b2 + b1) + tg
     float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
 
-    bool ok = true;
+    bool ok = true, k_ahead = false;                   // K of page `loaded` is on its way
     for (; active && used < it.num_pages; used += PG) {
         const int st = used % NS;
         if (!dev::mbar_wait_bounded(full + 8 * st, (used / NS) & 1, a.wait_limit_ns, nullptr)) {
@@ -166,6 +184,11 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
                 dev::f32x2_split(acc[r], lo, hi);
                 d[i][r] = lo + hi;
             }
+        }
+        if (split && loaded < it.num_pages) {
+            __syncwarp();
+            load(loaded, true, false);
+            k_ahead = true;
         }
         // sums over the 8 lanes, halving the (token, row) set each time
         float x[2];
@@ -218,6 +241,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
             p[h] = exp2f(x[h] - m[h]);
             l[h] += p[h];
         }
+        if (split && !dev::mbar_wait_bounded(vfull + 8 * st, (used / NS) & 1, a.wait_limit_ns, nullptr)) {
+            ok = false;
+            break;
+        }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             unsigned long long pr[kWarpRows];
@@ -248,7 +275,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
                 used += PG;
                 break;
             }
-            load(loaded);
+            load(loaded, !split, true);
+            k_ahead = false;
             loaded += PG;
         }
     }
@@ -259,8 +287,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         }
         // copies this warp issued must land before the CTA's shared memory goes
         if (rgi == 0)
-            for (int pg = used; pg < loaded; pg += PG)
-                dev::mbar_wait_bounded(full + 8 * (pg % NS), (pg / NS) & 1, kDrainNs, nullptr);
+            for (int pg = used; pg <= loaded && pg < it.num_pages; pg += PG) {
+                // k_ahead: the wait for V of page `used` failed, its K was read
+                // and K of page `loaded` may be on its way into the same stage
+                if (pg < loaded ? !(k_ahead && pg == used) : k_ahead)
+                    dev::mbar_wait_bounded(full + 8 * (pg % NS), (pg / NS) & 1, kDrainNs, nullptr);
+                if (pg < loaded && split)
+                    dev::mbar_wait_bounded(vfull + 8 * (pg % NS), (pg / NS) & 1, kDrainNs, nullptr);
+            }
     }
 
     // l over the tokens; o over the token groups, leaving lane group tg row tg
