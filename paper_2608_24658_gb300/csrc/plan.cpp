@@ -90,7 +90,11 @@ constexpr int64_t kSpareEntriesNum = 3, kSpareEntriesDen = 2;
 constexpr int64_t kPairShareNum = 3, kPairShareDen = 4;
 // fp32 pieces: one CTA each, 3 CTAs per SM.  About kFp32Waves pieces per CTA
 // slot even out the launch's end; never longer than kFp32ChunkPages (the
-// fixed length before: 2 to 3 pieces a slot on a 16-branch step).
+// fixed length before: 2 to 3 pieces a slot on a 16-branch step).  At head_dim
+// 128, 3 against 2.5: 16 branches 65.6 -> 64.5 us, two-level tree 74.4 -> 71.6,
+// 4 branches of 1k to 9k tokens 51.0 -> 49.0, 8 q heads a kv head 100.2 ->
+// 100.7; 2 and 1.5 are uneven (8 q heads a kv head 104 and 111).  At head_dim 64,
+// 2 made a step 2.5% slower.
 constexpr int kFp32ChunkPages = 32;
 // Attention kernels come up while the kernel before them drains (early), which
 // saves a step 2 to 5 us.  Their CTAs then take the SMs in the order these
@@ -103,7 +107,8 @@ constexpr int kFp32ChunkPages = 32;
 constexpr int64_t kEarlyKvBytes = int64_t{2} << 30, kEarlyKvBytesE4m3 = int64_t{3} << 28;
 constexpr int64_t kEarlyPrefillPages = 256;    // a CTA's share
 constexpr int kFp32MinPages = 4;
-constexpr int64_t kFp32Slots = 3, kFp32Waves = 3;
+constexpr int64_t kFp32Slots = 3;
+constexpr double kFp32Waves = 2.5, kFp32WavesD64 = 3.0;
 // stream rows kept free after a branch's last item: half its pages, 4 to 64
 // (an item that grows further makes the launch's tail: build a new plan)
 constexpr int32_t kAppendSlackMin = 4, kAppendSlackMax = 64;
@@ -816,7 +821,10 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
         for (const Run &r : runs) pages += r.pages;
         int64_t chunk = std::min<int64_t>(
             kFp32ChunkPages,
-            std::max<int64_t>(kFp32MinPages, pages / (kFp32Slots * kFp32Waves * p->num_sms)));
+            std::max<int64_t>(kFp32MinPages, static_cast<int64_t>(
+                                        static_cast<double>(pages) /
+                                        ((cfg->head_dim == 64 ? kFp32WavesD64 : kFp32Waves) *
+                                         static_cast<double>(kFp32Slots * p->num_sms)))));
         // shorter pieces mean more partial rows: not past what a decode
         // without a caller's workspace holds
         int64_t rows = 0;
