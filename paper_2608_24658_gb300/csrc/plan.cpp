@@ -69,14 +69,27 @@ constexpr double kMergePages = 28.0;
 constexpr double kLoneTileShare = 0.85;
 constexpr int kPieceCounts = 8;
 constexpr int kPrefillBlockPages = parason::kPrefillBoxPages;   // a prefill tile's blocks
-// suffix pieces: about this many per warp of the launch (at least
-// kMinPiecePages and at most kMaxPiecePages pages).  Same-box A/B against
-// 3: two-level step 79.7 -> 78.8 us, the Llama-3 shape level (its pieces
-// were at an 8-page floor); 2 made the Llama-3-shape step 2 us slower.
-// With e4m3 KV 2: two-level 64.5 -> 62.5 us, 8k prefix and 64 branches 71.0 ->
-// 68.3 (with bf16 KV slower: 16 branches 31.6 -> 33.0 us, and at head_dim 64
-// 16 x 16 branches 195 -> 205).
-constexpr double kNarrowPiecesPerWarp = 2.5, kNarrowPiecesPerWarpE4m3 = 2.0;
+// Suffix pieces: at most about kNarrowPiecesPerWarp per warp of the launch (and
+// kMinPiecePages to kMaxPiecePages pages); between that and one piece per warp,
+// the length whose queue ends first by a model of the pass (narrow_time): a
+// piece costs its pages and a start, every warp pulls the longest piece left,
+// and warps run at full speed only once fewer than a share of them is busy
+// (bf16 KV: HBM is then no longer full; e4m3 KV keeps them closer to their own
+// pace).  What decides is how the nodes' lengths divide: on 64 branches of 16
+// heads with e4m3 KV pieces of 41, 52, 65 and 83 pages took 131, 149, 128 and
+// 141 us.  Start and share were fitted to 16 trees at 10 to 13 lengths each;
+// the lengths chosen are within 2% (e4m3) and 1% (bf16) of the best of them, a
+// fixed 2 and 2.5 pieces per warp within 12% and 4%.
+// Against those: 16 branches 31.5 -> 30.2 us, two-level tree 69.3 -> 67.2, 4
+// requests x 32 branches at head_dim 64 42.0 -> 41.0; e4m3 KV 8k prefix and 64
+// branches 66.7 -> 63.4, 9 requests of 47 branches 128 -> 110 (slower: 64 branches
+// of a 16k prefix at head_dim 64 87.5 -> 90.2).  The choice takes no longer than
+// the items it saves (a plan of 1024 branches 8.4 -> 8.1 ms).
+constexpr double kNarrowPiecesPerWarp = 2.5;
+constexpr int64_t kNarrowStartPages = 2, kNarrowStartPagesE4m3 = 8;
+constexpr double kNarrowFullShare = 0.5, kNarrowFullShareE4m3 = 0.8;
+constexpr int kNarrowLengths = 10;         // lengths tried
+constexpr int64_t kNarrowTimeMax = 1 << 14;   // pages of a warp, where lengths matter little
 constexpr double kWideProvision = 1.15;   // prefix CTAs relative to the cost model
 // Decode: up to this many prefix queue entries per prefix CTA (num / den)
 // become one CTA each; up to two, two entries each
@@ -145,6 +158,45 @@ void piece_split(int64_t pages, int64_t chunk, int64_t align, int64_t &per, int6
     per = (pages + n - 1) / n;
     per = (per + align - 1) / align * align;
     n = (pages + per - 1) / per;
+}
+
+// The suffix pass of `lens` (pages of a run, runs of that length) in pieces of at
+// most `chunk` (<= kMaxPiecePages) pages, in pages of one warp: `early` warps from
+// time 0, `late` more from t_late on; below `full` busy warps time runs at
+// full speed.  Negative when it is longer than kNarrowTimeMax.
+double narrow_time(const std::vector<std::pair<int64_t, int64_t>> &lens, int64_t chunk, int64_t start,
+                   double full, int64_t early, int64_t late, int64_t t_late) {
+    int64_t pieces[kMaxPiecePages + 1] = {};
+    int64_t work = 0;
+    for (const auto &l : lens) {
+        int64_t per = 0, n = 0;
+        piece_split(l.first, chunk, 1, per, n);
+        pieces[per] += (n - 1) * l.second;
+        pieces[l.first - per * (n - 1)] += l.second;
+        work += (l.first + n * start) * l.second;
+    }
+    const int64_t horizon = work / std::max<int64_t>(1, early) + t_late + kMaxPiecePages + start + 2;
+    if (horizon > kNarrowTimeMax) return -1.0;
+    // warps that are next free at each time
+    std::vector<int64_t> free_at(static_cast<size_t>(horizon + kMaxPiecePages + start), 0);
+    free_at[0] += early;
+    free_at[static_cast<size_t>(t_late)] += late;
+    size_t t = 0;
+    for (int64_t size = kMaxPiecePages; size > 0; --size)
+        while (pieces[size] > 0) {
+            while (free_at[t] == 0) ++t;
+            const int64_t k = std::min(pieces[size], free_at[t]);
+            free_at[t] -= k;
+            free_at[t + static_cast<size_t>(size + start)] += k;
+            pieces[size] -= k;
+        }
+    double end = 0.0;
+    int64_t busy = early + late;
+    for (size_t u = 0; u < free_at.size() && busy > 0; ++u) {
+        busy -= free_at[u];
+        end += std::max(1.0, static_cast<double>(busy) / full) * (busy > 0 ? 1.0 : 0.0);
+    }
+    return end;
 }
 
 // A prefill's runs of one (chunk, kv head, page list): its pages, tiles and rows.
@@ -840,12 +892,46 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
             if (!cut(r, chunk, 1)) return PARASON_EUNSUPPORTED;
     } else {
         const int64_t total_warps = static_cast<int64_t>(p->num_sms) * p->suffix_warps;
-        const double pieces = mode == PARASON_FP8_E4M3_KV ? kNarrowPiecesPerWarpE4m3 : kNarrowPiecesPerWarp;
-        const int64_t narrow_chunk = std::min<int64_t>(
-            kMaxPiecePages,
-            std::max<int64_t>(kMinPiecePages,
-                              static_cast<int64_t>(static_cast<double>(narrow_pages) /
-                                                   (pieces * std::max<int64_t>(1, total_warps)))));
+        const double share = static_cast<double>(narrow_pages) /
+                             static_cast<double>(std::max<int64_t>(1, total_warps));
+        auto length_at = [&](double pieces) {
+            return std::min<int64_t>(kMaxPiecePages,
+                                     std::max<int64_t>(kMinPiecePages, static_cast<int64_t>(share / pieces)));
+        };
+        int64_t narrow_chunk = length_at(kNarrowPiecesPerWarp);
+        if (n_narrow_ctas > 0 && length_at(1.0) > narrow_chunk) {
+            const bool e4m3 = mode == PARASON_FP8_E4M3_KV;
+            std::vector<std::pair<int64_t, int64_t>> lens;
+            for (const Run &r : runs)
+                if (!r.wide && r.pages > 0) {
+                    if (!lens.empty() && lens.back().first == r.pages)
+                        ++lens.back().second;
+                    else
+                        lens.emplace_back(r.pages, 1);
+                }
+            const int64_t early = static_cast<int64_t>(n_narrow_ctas) * p->suffix_warps;
+            const int64_t late = static_cast<int64_t>(n_wide) * p->suffix_warps;
+            const int64_t t_late = late > 0 ? static_cast<int64_t>(wide_cost / static_cast<double>(late)) : 0;
+            const double full =
+                (e4m3 ? kNarrowFullShareE4m3 : kNarrowFullShare) * static_cast<double>(early + late);
+            double best = 0.0;
+            int64_t tried = 0, pick = narrow_chunk;
+            for (int c = 0; c <= kNarrowLengths; ++c) {
+                const double pieces = kNarrowPiecesPerWarp *
+                                      std::pow(1.0 / kNarrowPiecesPerWarp, static_cast<double>(c) / kNarrowLengths);
+                const int64_t length = length_at(pieces);
+                if (length == tried) continue;
+                tried = length;
+                const double t = narrow_time(lens, length, e4m3 ? kNarrowStartPagesE4m3 : kNarrowStartPages,
+                                             full, early, late, t_late);
+                if (t < 0.0) break;
+                if (best == 0.0 || t < best) {
+                    best = t;
+                    pick = length;
+                }
+            }
+            narrow_chunk = pick;
+        }
         p->narrow_chunk = narrow_chunk;
         if (prefill && n_wide > 0 && !runs.empty()) {
             std::vector<PrefillGroup> groups;
