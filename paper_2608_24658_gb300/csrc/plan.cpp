@@ -133,8 +133,8 @@ constexpr double kTcPageCost = 2.0;          // one page of a tcgen05 prefix til
 // of a 2k prefix over 16 branches 76.7, 76.7, 80.6; 2.6 and the start 184 and
 // 77.1; a 32k prefix over 128 branches of 4k to 16k 521, 521, 506)
 constexpr double kTcPageCostE4m3 = 2.6;
-// (a quarter of a short tile: with all 24 pages, tiles of 5 to 30 pages got more
-// CTAs than they fill and were cut for them, 16.2 -> 23.4 us and 21.3 -> 28.0)
+// (a third of a short tile: with all 24 pages, tiles of 5 to 30 pages got more
+// CTAs than they fill and were cut for them, 16.7 -> 23.4 us and 21.3 -> 28.0)
 constexpr int64_t kTcStartPagesE4m3 = 24;
 constexpr double kTcPageCostD64 = 2.5;       // the same at head_dim 64 (tuned: 16 requests x 16
                                              // branches 201.1, 196.5, 196.5 us at 2.0, 2.5, 3.0;
@@ -672,7 +672,7 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
                 if (wide)
                     wide_cost += run.cost_per_page *
                                  static_cast<double>(P + (mode == PARASON_FP8_E4M3_KV
-                                                              ? std::min<int64_t>(kTcStartPagesE4m3, P / 4)
+                                                              ? std::min<int64_t>(kTcStartPagesE4m3, P / 3)
                                                               : 0));
                 else
                     narrow_pages += P;
