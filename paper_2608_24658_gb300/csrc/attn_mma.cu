@@ -19,7 +19,7 @@
 //        from shared memory; 4 softmax warps own one row per thread (TMEM
 //        lane) and write P over S; 4 epilogue warps store an item's O and
 //        load Q two items ahead (with e4m3 KV they also convert each staged
-//        block to f16).
+//        block to f16, and load an item's Q before its first block).
 //      - bf16 at head_dim 128, when the planner pairs row tiles: two
 //        128-row tiles of a piece against each staged block
 //        (prefix_cta_tc_pair), Q in shared memory, each tile's S/P and O in
@@ -29,8 +29,9 @@
 //    an independent worker with its own TMA ring that pulls split-K pieces
 //    from a queue: no CTA barrier, no cross-warp combine.  QK^T and PV are
 //    mma.sync m16n8k16 with fp32 accumulation and a quad-shuffle online
-//    softmax; tiles of 5 to 8 rows run the transposed step (S^T = K Q^T),
-//    with e4m3 KV two pages per softmax update.  A bf16 page at head_dim 128
+//    softmax; tiles of 5 to 8 rows (at head_dim 64 of up to 8) run the
+//    transposed step (S^T = K Q^T), with e4m3 KV or at head_dim 64 two pages
+//    per softmax update.  A bf16 page at head_dim 128
 //    comes in one TMA box per tensor (the 4-D page maps).
 //
 // Every item writes a partial (o, m, l) per row.  The merge kernel (merge.cu)
@@ -1117,8 +1118,7 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
         // ------------------------------------------------------------ producer
         const bool skip_first = a.debug_flags & PARASON_DEBUG_SKIP_FIRST_LOAD;
         // bf16 KV: the tile's K and V go to L2 as evict-last (measured: the
-        // Llama-3-shape step 42.9 -> 41.4 us, the long-prefix one -1 us, the
-        // join prefill +1%; no gain with e4m3 KV, which keeps the default)
+        // Llama-3-shape step 42.9 -> 41.4 us, the long-prefix one -1 us; no gain with e4m3 KV, which keeps the default)
         const uint64_t last_pol = dev::l2_evict_last_policy();
         // e4m3 blocks keep the default L2 policy (the per-page boxes use no hint)
         const uint64_t f8_pol = dev::l2_evict_normal_policy();
