@@ -67,7 +67,16 @@ constexpr double kPieceStartPages = 28.0;
 constexpr double kPiecePartialPages = 39.0;
 constexpr double kMergePages = 28.0;
 constexpr double kLoneTileShare = 0.85;
+// With e4m3 KV a page takes kPrefillPageE4m3 of that, since its chain is longer
+// (1.0 and 1.7: an 816-token prefix and one short chunk of 16 heads 19.9 and
+// 12.5 us, here 12.5; two chunks under a 4k prefix 107 and 123, here 107).
+constexpr double kPrefillPageE4m3 = 1.35;
 constexpr int kPieceCounts = 8;
+// With e4m3 KV a prefill of up to this many pairs per SM reads whole paths
+// (one list of pages per pair and kv head, as with bf16 KV), of more a run per
+// node: join prefill 796 -> 664 us, fork 78.9 -> 54.2, 30 chunks of 2 to 5 tokens
+// with 16 kv heads (3.2 pairs an SM) 42.2 -> 25.2.
+constexpr int64_t kListPairsE4m3 = 4;
 constexpr int kPrefillBlockPages = parason::kPrefillBoxPages;   // a prefill tile's blocks
 // Suffix pieces: at most about kNarrowPiecesPerWarp per warp of the launch (and
 // kMinPiecePages to kMaxPiecePages pages); between that and one piece per warp,
@@ -215,7 +224,7 @@ struct PrefillGroup {
 // + 1 of them a whole piece more than those that take n, where long pieces
 // and remainders even out with the fewest pieces.
 double prefill_queue_time(const std::vector<PrefillGroup> &groups, int64_t chunk, int32_t ctas,
-                          bool whole_paths, int64_t &rows) {
+                          bool whole_paths, double page, int64_t &rows) {
     std::vector<std::pair<int64_t, double>> entries;   // (pages, time)
     rows = 0;
     bool whole = true;                                 // no group is cut
@@ -225,8 +234,8 @@ double prefill_queue_time(const std::vector<PrefillGroup> &groups, int64_t chunk
             const int64_t np = std::min(left, chunk);
             left -= np;
             rows += g.rows;
-            const double t = static_cast<double>((np + kPrefillBlockPages - 1) / kPrefillBlockPages *
-                                                 kPrefillBlockPages);
+            const double t = page * static_cast<double>((np + kPrefillBlockPages - 1) / kPrefillBlockPages *
+                                                        kPrefillBlockPages);
             for (int32_t k = 0; k < g.tiles / 2; ++k) entries.emplace_back(np, t + kPieceStartPages);
             if (g.tiles % 2) entries.emplace_back(np, kLoneTileShare * t + kPieceStartPages);
         }
@@ -254,7 +263,7 @@ double prefill_queue_time(const std::vector<PrefillGroup> &groups, int64_t chunk
 // whose partial rows pass what a decode without a caller's workspace holds is
 // taken only if none stays under it.
 int64_t prefill_cut(const std::vector<PrefillGroup> &groups, int32_t ctas, bool whole_paths,
-                    int64_t max_rows) {
+                    double page, int64_t max_rows) {
     int64_t longest = 0, total = 0;
     for (const PrefillGroup &g : groups) {
         longest = std::max(longest, g.pages);
@@ -276,7 +285,7 @@ int64_t prefill_cut(const std::vector<PrefillGroup> &groups, int32_t ctas, bool 
     bool best_fits = false;
     for (int64_t c : cands) {
         int64_t rows = 0;
-        const double t = prefill_queue_time(groups, c, ctas, whole_paths, rows);
+        const double t = prefill_queue_time(groups, c, ctas, whole_paths, page, rows);
         const bool fits = rows <= max_rows;
         if (best_t < 0.0 || (fits && !best_fits) || (fits == best_fits && t < best_t)) {
             best = c;
@@ -552,7 +561,16 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
     std::vector<Run> runs;
     int64_t narrow_pages = 0;
     double wide_cost = 0.0;
+    bool lists = false;               // a prefill's runs are whole paths
     if (prefill) {
+        int64_t pairs = 0;
+        for (int32_t c = 0; c < num_leaves; ++c) {
+            const int64_t R = static_cast<int64_t>(node_len[leaf_node[c]]) * g;
+            const int64_t rt = std::max(1, tile_rows_for(static_cast<int32_t>(std::min<int64_t>(R, 1 << 20)), g, mode));
+            pairs += H_kv * ((R + 2 * rt - 1) / (2 * rt));
+        }
+        lists = cfg->head_dim == 128 &&
+                (mode == PARASON_BF16 || pairs <= kListPairsE4m3 * static_cast<int64_t>(p->num_sms));
         // chunk c: rows (token t, q head r) = t * g + r of every kv head, in
         // tiles that run in pairs; each pair reads every ancestor in full and
         // its own node up to the pair's last token
@@ -566,7 +584,7 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
             std::vector<int32_t> path;
             for (int32_t m = n; m >= 0; m = parent[m]) path.push_back(m);
             std::reverse(path.begin(), path.end());
-            if (mode == PARASON_BF16 && cfg->head_dim == 128) {
+            if (lists) {
                 // one list per tile pair, up to the pair's last token; a pair's
                 // first tile reads the few pages past its own last token masked
                 const int64_t pair_rows = 2 * static_cast<int64_t>(rt);
@@ -605,7 +623,7 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
                             run.span = si;
                             run.leaf_lo = qbase[c];
                             run.wide = true;
-                            run.cost_per_page = wide_page_cost(cfg->head_dim, false);
+                            run.cost_per_page = wide_page_cost(cfg->head_dim, mode == PARASON_FP8_E4M3_KV);
                             wide_cost += run.cost_per_page * static_cast<double>(run.pages);
                             runs.push_back(run);
                         }
@@ -948,7 +966,7 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
             }
             const int64_t row_bytes = static_cast<int64_t>(cfg->head_dim) * 4 + 8;
             wide_chunk = prefill_cut(
-                groups, n_wide, mode == PARASON_BF16,   // (e4m3 runs are one node's)
+                groups, n_wide, lists, mode == PARASON_BF16 ? 1.0 : kPrefillPageE4m3,
                 (PARASON_NO_ALLOC_SCRATCH_BYTES - 2 * static_cast<int64_t>(kAlign)) / row_bytes);
         }
         // The row tiles of one (node, kv head) read the same pages: their

@@ -39,7 +39,7 @@ def test_prefill_tile_and_block_edges(mode, permute):
                            list(range(n, 2 * n)), num_q_heads=8, num_kv_heads=2, head_dim=128,
                            mode=mode, seed=3, permute_pages=permute, extra_pages=5,
                            tail_value=float("nan"), q_std=0.35, device="cuda")
-    check(tree, whole=mode == "bf16")
+    check(tree)
 
 
 @pytest.mark.parametrize("mode", ["bf16", "fp8"])
@@ -77,3 +77,12 @@ def test_prefill_whole_paths_write_the_result():
         again, none = plan.decode_tree(tree, want_lse=False)
         plan.check()
     assert none is None and torch.equal(out, again)
+
+
+def test_prefill_e4m3_many_pairs():
+    """More than 4 tile pairs per SM with e4m3 KV: a run per node, not whole paths."""
+    n = 4 * torch.cuda.get_device_properties(0).multi_processor_count // 16 + 2
+    tree = W.build_prefill("many", [-1, 0] + [1] * n, [70, 9] + [1 + k % 3 for k in range(n)],
+                           list(range(2, 2 + n)), num_q_heads=16, num_kv_heads=16, head_dim=128,
+                           mode="fp8", seed=6, q_std=0.35, tail_value=float("nan"), device="cuda")
+    check(tree, whole=False)
