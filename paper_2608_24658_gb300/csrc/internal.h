@@ -137,6 +137,9 @@ cudaError_t attn_mma_ctas_per_sm(int head_dim, int mode, int *ctas_per_sm);
 // have their 8-row groups 2 KB apart, v as the decode plan's page box.
 constexpr int kTcRunPages = 4;
 constexpr int kDecodeBoxPages = 1, kPrefillBoxPages = 8;
+// A prefill CTA's pairs in flight, and the blocks in pairs that it pulls ahead of
+// the producer (the planner simulates the same rule).
+constexpr int kPrefillMeta = 4, kPrefillAheadBlocks = 4;
 struct KvMaps {
     CUtensorMap k, v, k_run, v_run, k_box, v_box;
 };

@@ -16,6 +16,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <limits>
 #include <mutex>
 #include <new>
 #include <queue>
@@ -56,21 +57,29 @@ constexpr int kWideBlockPages = 4;      // prefix pieces are whole 64-token bloc
 constexpr int64_t kWidePiecesPerCta = 1;
 // A prefill's queue is the whole launch, and nothing evens out its CTAs' ends:
 // its piece length is the one, of a few candidates, under which the queue,
-// simulated, empties first (prefill_cut).  In pages of a pair (0.21 us with
-// bf16 KV): an entry's start and its O cost a CTA kPieceStartPages (43-block
-// pieces took 82 us where 281-block ones took 1.67 us a block); its partial
-// rows, written and read back by the merge, every CTA another
-// kPiecePartialPages / num_sms; the merge itself kMergePages, unless every
-// entry holds its rows' whole paths; a pair without a second tile takes
-// kLoneTileShare of a pair's time.
-constexpr double kPieceStartPages = 28.0;
-constexpr double kPiecePartialPages = 39.0;
-constexpr double kMergePages = 28.0;
-constexpr double kLoneTileShare = 0.85;
-// With e4m3 KV a page takes kPrefillPageE4m3 of that, since its chain is longer
-// (1.0 and 1.7: an 816-token prefix and one short chunk of 16 heads 19.9 and
-// 12.5 us, here 12.5; two chunks under a 4k prefix 107 and 123, here 107).
-constexpr double kPrefillPageE4m3 = 1.35;
+// simulated, empties first (prefill_cut).  In pages of a pair with bf16 KV (0.21
+// us): a page takes `page` (with e4m3 KV the tiles' chain is longer), a pair
+// without a second tile `lone` of a pair's time; an entry costs its CTA `start`
+// and, unless it writes the result, kEntryRowPages a row for its partials; a
+// merge, unless every entry holds its rows' whole paths, costs `merge`, and every
+// CTA its share of the partial rows, written and read back, and of the result's
+// rows.  The CTAs pull as the kernel's scheduler does, kPullPages apart and
+// kPullLeadBlocks before a pair's end: those with short pairs take several at
+// once, so that a queue a little longer than the CTAs ends late (64 pairs of 144
+// to 185 pages cut into 176 entries take 53 us, into 128 43).
+// Fitted to 475 prefills (1 to 32 chunks of 1 to 4096 tokens over paths of up to
+// 30k, seven head groups, both KV formats) at up to 32 cuts each: the cuts taken
+// are 0.5% off the best measured, against 2.5% with a charge for partials by the
+// entry, whatever its rows (39 pages, and 28 for the merge), which left short
+// chunks whole: 4 x 33 tokens under a 2k prefix, 16 kv heads, 32.6 us whole and
+// 22.8 in two pieces.
+struct PrefillCost {
+    double page, lone, start, merge;
+};
+constexpr PrefillCost kPrefillBf16 = {1.0, 0.95, 20.0, 12.0};
+constexpr PrefillCost kPrefillE4m3 = {1.35, 0.85, 36.0, 8.0};
+constexpr double kEntryRowPages = 0.01, kPartialRowPages = 0.12, kOutRowPages = 0.15;
+constexpr double kPullPages = 7.0, kPullLeadBlocks = 6.0;
 constexpr int kPieceCounts = 8;
 // With e4m3 KV a prefill of up to this many pairs per SM reads whole paths
 // (one list of pages per pair and kv head, as with bf16 KV), of more a run per
@@ -216,45 +225,91 @@ struct PrefillGroup {
     int32_t tiles, rows;
 };
 
+// When, in pages, a CTA that has pulled `n` pairs pulls the next: the rule of
+// the kernel's scheduler warp, with `nb` and `end` the blocks and the ends of its
+// last kPrefillMeta pairs (the newest first) and `block` the time of a block.
+double next_pull(int n, const int (&nb)[parason::kPrefillMeta], const double (&end)[parason::kPrefillMeta],
+                 double last, double block) {
+    int back = 0;                                      // pairs the producer need not be through
+    for (int blocks = 0; back < n && back < parason::kPrefillMeta - 1; ++back) {
+        blocks += nb[back];
+        if (blocks > parason::kPrefillAheadBlocks) break;
+    }
+    return std::max(last + kPullPages, back < n ? end[back] - kPullLeadBlocks * block : 0.0);
+}
+
 // Time, in pages, for `ctas` CTAs to empty a prefill queue whose groups are
-// cut into pieces of `chunk` pages, and the partial rows that takes.  The
+// cut into pieces of `chunk` pages, and the partial rows that takes (for more than
+// `exact_rows` of those, an even split of the work if that reaches `limit`).  The
 // queue hands its pairs out longest first, the first `ctas` to the CTAs that
-// own them, each later one to the CTA that frees first.  A run is cut into
+// own them, each later one to the CTA that pulls first.  A run is cut into
 // whole pieces and a remainder: equal pieces would give the CTAs that take n
 // + 1 of them a whole piece more than those that take n, where long pieces
 // and remainders even out with the fewest pieces.
 double prefill_queue_time(const std::vector<PrefillGroup> &groups, int64_t chunk, int32_t ctas,
-                          bool whole_paths, double page, int64_t &rows) {
+                          bool whole_paths, const PrefillCost &cost, int64_t out_rows,
+                          int64_t exact_rows, double limit, int64_t &rows) {
     std::vector<std::pair<int64_t, double>> entries;   // (pages, time)
     rows = 0;
-    bool whole = true;                                 // no group is cut
-    for (const PrefillGroup &g : groups)
+    size_t n = 0;
+    bool whole = whole_paths;                          // no group is cut, and no CTA has two entries
+    for (const PrefillGroup &g : groups) {
+        whole = whole && g.pages <= chunk;
+        n += static_cast<size_t>((g.tiles + 1) / 2);
+    }
+    whole = whole && n <= static_cast<size_t>(ctas);
+    const double block = cost.page * kPrefillBlockPages;
+    auto blocks_of = [](int64_t pages) { return (pages + kPrefillBlockPages - 1) / kPrefillBlockPages; };
+    for (const PrefillGroup &g : groups) {
+        const double start = cost.start + (whole ? 0.0 : kEntryRowPages * g.rows / ((g.tiles + 1) / 2));
         for (int64_t left = g.pages; left > 0;) {
-            whole = whole && left <= chunk;
             const int64_t np = std::min(left, chunk);
             left -= np;
             rows += g.rows;
-            const double t = page * static_cast<double>((np + kPrefillBlockPages - 1) / kPrefillBlockPages *
-                                                        kPrefillBlockPages);
-            for (int32_t k = 0; k < g.tiles / 2; ++k) entries.emplace_back(np, t + kPieceStartPages);
-            if (g.tiles % 2) entries.emplace_back(np, kLoneTileShare * t + kPieceStartPages);
+            const double t = block * static_cast<double>(blocks_of(np));
+            for (int32_t k = 0; k < g.tiles / 2; ++k) entries.emplace_back(np, start + t);
+            if (g.tiles % 2) entries.emplace_back(np, start + cost.lone * t);
         }
+    }
+    double merge = 0.0;
+    if (!whole)
+        merge = cost.merge +
+                (kPartialRowPages * static_cast<double>(rows) + kOutRowPages * static_cast<double>(out_rows)) / ctas;
+    double work = 0.0;
+    for (const auto &e : entries) work += e.second;
+    if (rows > exact_rows && work / ctas + merge >= limit) return work / ctas + merge;
     std::stable_sort(entries.begin(), entries.end(),
                      [](const auto &a, const auto &b) { return a.first > b.first; });
-    std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+    struct Cta {
+        int n = 0, nb[parason::kPrefillMeta] = {};     // pairs so far, and of the last ones ...
+        double end[parason::kPrefillMeta] = {};        // ... the blocks and the ends
+    };
+    const size_t owned = std::min(entries.size(), static_cast<size_t>(ctas));
+    std::vector<Cta> cta(owned);
+    std::priority_queue<std::pair<double, size_t>, std::vector<std::pair<double, size_t>>,
+                        std::greater<std::pair<double, size_t>>> pulls;   // (time of the next, CTA)
     double end = 0.0;
-    for (size_t e = 0; e < entries.size(); ++e) {
+    for (size_t i = 0; i < entries.size(); ++i) {
         double t0 = 0.0;
-        if (e >= static_cast<size_t>(ctas)) {
-            t0 = free_at.top();
-            free_at.pop();
+        size_t c = i;
+        if (i >= owned) {
+            t0 = pulls.top().first;
+            c = pulls.top().second;
+            pulls.pop();
         }
-        const double t1 = t0 + entries[e].second;
-        free_at.push(t1);
+        Cta &x = cta[c];
+        const double t1 = std::max(t0, x.end[0]) + entries[i].second;
+        for (int k = parason::kPrefillMeta - 1; k > 0; --k) {
+            x.nb[k] = x.nb[k - 1];
+            x.end[k] = x.end[k - 1];
+        }
+        x.nb[0] = static_cast<int>(blocks_of(entries[i].first));
+        x.end[0] = t1;
+        ++x.n;
         end = std::max(end, t1);
+        if (owned < entries.size()) pulls.emplace(next_pull(x.n, x.nb, x.end, t0, block), c);
     }
-    if (whole && whole_paths && entries.size() <= static_cast<size_t>(ctas)) return end;
-    return end + kMergePages + kPiecePartialPages * static_cast<double>(entries.size()) / ctas;
+    return end + merge;
 }
 
 // The piece length of a prefill plan.  Candidates: the longest run cut into n
@@ -263,7 +318,7 @@ double prefill_queue_time(const std::vector<PrefillGroup> &groups, int64_t chunk
 // whose partial rows pass what a decode without a caller's workspace holds is
 // taken only if none stays under it.
 int64_t prefill_cut(const std::vector<PrefillGroup> &groups, int32_t ctas, bool whole_paths,
-                    double page, int64_t max_rows) {
+                    const PrefillCost &cost, int64_t out_rows, int64_t max_rows) {
     int64_t longest = 0, total = 0;
     for (const PrefillGroup &g : groups) {
         longest = std::max(longest, g.pages);
@@ -285,7 +340,9 @@ int64_t prefill_cut(const std::vector<PrefillGroup> &groups, int32_t ctas, bool 
     bool best_fits = false;
     for (int64_t c : cands) {
         int64_t rows = 0;
-        const double t = prefill_queue_time(groups, c, ctas, whole_paths, page, rows);
+        const double t = prefill_queue_time(groups, c, ctas, whole_paths, cost, out_rows,
+                                            best_fits ? 0 : max_rows,
+                                            best_t < 0.0 ? std::numeric_limits<double>::infinity() : best_t, rows);
         const bool fits = rows <= max_rows;
         if (best_t < 0.0 || (fits && !best_fits) || (fits == best_fits && t < best_t)) {
             best = c;
@@ -966,7 +1023,8 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
             }
             const int64_t row_bytes = static_cast<int64_t>(cfg->head_dim) * 4 + 8;
             wide_chunk = prefill_cut(
-                groups, n_wide, lists, mode == PARASON_BF16 ? 1.0 : kPrefillPageE4m3,
+                groups, n_wide, lists, mode == PARASON_BF16 ? kPrefillBf16 : kPrefillE4m3,
+                static_cast<int64_t>(p->num_leaves) * cfg->num_q_heads,
                 (PARASON_NO_ALLOC_SCRATCH_BYTES - 2 * static_cast<int64_t>(kAlign)) / row_bytes);
         }
         // The row tiles of one (node, kv head) read the same pages: their

@@ -82,8 +82,8 @@ constexpr int kPagedBytes = kSlotBytes / kBlockPages;          // 4 KB: a page o
 constexpr int kRawSlotBytes = kBlockTokens * 128;              // 16 KB: the same in e4m3
 constexpr int kQColBlockBytes = kRows * 128;                   // 16 KB
 constexpr int kQBytes = 2 * kQColBlockBytes;                   // 32 KB a tile
-constexpr int kMeta = 4;
-constexpr int kAheadBlocks = 4;                    // (see the scheduler)
+constexpr int kMeta = kPrefillMeta;
+constexpr int kAheadBlocks = kPrefillAheadBlocks;  // (see the scheduler)
 constexpr int kValidRing = 8;
 constexpr uint32_t kTmemO = 0, kTmemS = 256;
 constexpr int kTmemCols = 512;
