@@ -112,6 +112,8 @@ constexpr double kWideProvision = 1.15;   // prefix CTAs relative to the cost mo
 // Decode: up to this many prefix queue entries per prefix CTA (num / den)
 // become one CTA each; up to two, two entries each
 constexpr int64_t kSpareEntriesNum = 3, kSpareEntriesDen = 2;
+// a lengthened piece takes at most this many times an SM's share of the pass
+constexpr double kLongestPiece = 2.25;
 // pairs of tcgen05 row tiles when at least this share of the prefix
 // tile-pages sits in pieces of two or more tiles.  Same-box A/B, pairs
 // against single tiles: 32k prefix tile alone 207.4 -> 155.8 us, join
@@ -849,13 +851,26 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
             // one each would take too many SMs: longer pieces, at most as
             // many as CTAs (16k prefix and 64 branches at head_dim 64: 96
             // entries on 75 CTAs 109.7 us, 64 on 64 87.8 us; 8k and 64 branches
-            // with e4m3 KV 84.7 -> 71.4 us)
-            int64_t chunk = wide_chunk, e = entries;
+            // with e4m3 KV 84.7 -> 71.4 us), unless short nodes hold the CTAs
+            // and a long one's piece would outlast the rest of the pass (4k
+            // prefix, 8 nodes of 64 tokens, 16 branches each: 75.6 us with whole
+            // 256-page tile pairs, 42.5 with pieces of 86; of trees whose
+            // pieces take up to 1.8 times an SM's share of the pass all gained,
+            // up to 17%, and from 2.8 times on all lost)
+            int64_t chunk = wide_chunk, e = entries, longest = 0;
             while (e > n_wide && chunk < kMaxTileItemPages) {
                 chunk = std::min<int64_t>(kMaxTileItemPages, chunk + kWideBlockPages);
                 e = entries_at(chunk);
             }
-            if (e <= n_wide) {
+            for (const Run &r : runs)
+                if (r.wide) {
+                    int64_t per = 0, n = 0;
+                    piece_split(r.pages, chunk, kWideBlockPages, per, n);
+                    longest = std::max(longest, std::min(per, r.pages));
+                }
+            const double piece = static_cast<double>(longest * (p->tc_pairs ? 2 : 1)) *
+                                 wide_page_cost(cfg->head_dim, mode == PARASON_FP8_E4M3_KV);
+            if (e <= n_wide && piece * S <= kLongestPiece * (wide_cost + static_cast<double>(narrow_pages))) {
                 wide_chunk = chunk;
                 n_wide = static_cast<int32_t>(e);
                 n_narrow_ctas = S - n_wide;
