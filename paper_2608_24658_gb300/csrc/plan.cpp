@@ -109,6 +109,19 @@ constexpr double kNarrowFullShare = 0.5, kNarrowFullShareE4m3 = 0.8;
 constexpr int kNarrowLengths = 10;         // lengths tried
 constexpr int64_t kNarrowTimeMax = 1 << 14;   // pages of a warp, where lengths matter little
 constexpr double kWideProvision = 1.15;   // prefix CTAs relative to the cost model
+// A prefix tile's start and its O take a CTA 3.5 us (head_dim 64) to 5 us, which
+// the costs by the page leave out: tiles of up to kShortTilePages pages each in the
+// mean, kShortTilesPerCta or more to a CTA, are charged kTileStartPages more and
+// get CTAs to be through with the rest of the pass, or within kShortPassPages (a
+// pass of 15 us or less, where the CTAs are wanted for its one round of suffix
+// pieces: 24 tiles on 24 CTAs for 11, 16.6 -> 21.6 us); at most one an entry, and
+// half of all.  Without, a one-page prefix of 64 branches of 500 tokens, 64 q / 8
+// kv heads, ran its 32 tiles on one CTA: 116 -> 20 us at head_dim 64, 156 -> 30 with
+// e4m3 KV; 8 requests x 32 branches under 64 tokens 70 -> 33 and 77 -> 44.  Between
+// 30 and 50 pages the times are level; longer tiles, charged so, are up to 20%
+// slower on more CTAs.
+constexpr int64_t kShortTilePages = 8, kShortTilesPerCta = 3;
+constexpr double kTileStartPages = 40.0, kShortPassPages = 120.0;
 // Decode: up to this many prefix queue entries per prefix CTA (num / den)
 // become one CTA each; up to two, two entries each
 constexpr int64_t kSpareEntriesNum = 3, kSpareEntriesDen = 2;
@@ -878,6 +891,24 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
         } else if (entries > n_wide && !one_each && entries <= 2 * static_cast<int64_t>(n_wide)) {
             n_wide = static_cast<int32_t>((entries + 1) / 2);
             n_narrow_ctas = S - n_wide;
+        }
+        // short tiles: their starts, not their pages, are a prefix CTA's time
+        int64_t tiles = 0;
+        for (const Run &r : runs)
+            if (r.wide) {
+                int64_t per = 0, n = 0;
+                piece_split(r.pages, wide_chunk, kWideBlockPages, per, n);
+                tiles += n;
+            }
+        if (wide_units <= kShortTilePages * tiles && entries >= kShortTilesPerCta * n_wide) {
+            const double cost = wide_cost + kTileStartPages * static_cast<double>(tiles);
+            const double pass = std::max(kShortPassPages, (cost + static_cast<double>(narrow_pages)) / S);
+            const int64_t want = std::min<int64_t>(
+                {static_cast<int64_t>(std::ceil(kWideProvision * cost / pass)), entries, S / 2});
+            if (want > n_wide) {
+                n_wide = static_cast<int32_t>(want);
+                n_narrow_ctas = S - n_wide;
+            }
         }
     }
     p->num_wide_ctas = n_wide;
