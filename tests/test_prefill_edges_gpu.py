@@ -29,16 +29,27 @@ def check(tree, whole=None):
     PT.compare(tree, out, lse, ref_o, ref_l, None, tree.name)
 
 
-@pytest.mark.parametrize("permute", [False, True])
-@pytest.mark.parametrize("mode", ["bf16", "fp8"])
-def test_prefill_tile_and_block_edges(mode, permute):
+def edges_tree(mode, permute=False):
     prefixes = [1, 63, 64, 65, 127, 128, 129, 300]
     chunks = [1, 31, 32, 33, 63, 64, 65, 2]
     n = len(prefixes)
-    tree = W.build_prefill("edges", [-1] * n + list(range(n)), prefixes + chunks,
+    return W.build_prefill("edges", [-1] * n + list(range(n)), prefixes + chunks,
                            list(range(n, 2 * n)), num_q_heads=8, num_kv_heads=2, head_dim=128,
                            mode=mode, seed=3, permute_pages=permute, extra_pages=5,
                            tail_value=float("nan"), q_std=0.35, device="cuda")
+
+
+def fork_tree(mode):
+    """9 chunks of 70 tokens, 32 q / 8 kv heads: 144 pairs, every other of 6 tokens."""
+    return W.build_prefill("fork", [-1] + [0] * 9, [100] + [70] * 9, list(range(1, 10)),
+                           num_q_heads=32, num_kv_heads=8, head_dim=128, mode=mode, seed=8,
+                           q_std=0.35, device="cuda")
+
+
+@pytest.mark.parametrize("permute", [False, True])
+@pytest.mark.parametrize("mode", ["bf16", "fp8"])
+def test_prefill_tile_and_block_edges(mode, permute):
+    tree = edges_tree(mode, permute)
     check(tree)
 
 
@@ -65,18 +76,29 @@ def test_prefill_growing_maxima(mode):
     check(tree)
 
 
-def test_prefill_whole_paths_write_the_result():
-    """Without a cut the attention kernel is the only launch; lse may be left out."""
-    tree = W.fork_prefill(device="cuda", chunk=5, threads=3)
+@pytest.mark.parametrize("name,mode", [("edges", "bf16"), ("fork", "bf16"), ("fork", "fp8")])
+def test_prefill_whole_paths_write_the_result(name, mode):
+    """Every pair whole and on a CTA of its own: the attention kernel is the only
+    launch.  Several calls on other q, one after the other and one without lse
+    (no merge sets the queue counters back between them), each against the
+    oracle."""
+    tree = edges_tree(mode) if name == "edges" else fork_tree(mode)
     with Plan.for_prefill(tree) as plan:
-        info = plan.info()
+        assert plan.launches_per_decode() == 1
         mrng = plan.export(_lib.TABLE_MERGE_RANGES)
-        single = bool((mrng[:, 1] - mrng[:, 0] == 1).all())
-        assert plan.launches_per_decode() == (1 if single and info["num_wide_items"] <= 2 * info["num_ctas"] else 2)
-        out, lse = plan.decode_tree(tree)
-        again, none = plan.decode_tree(tree, want_lse=False)
+        assert (mrng[:, 1] - mrng[:, 0] == 1).all()
+        q0, got = tree.q.clone(), []
+        for k, want_lse in enumerate((True, False, True)):
+            tree.q.copy_(q0.roll(k, dims=0))
+            got.append(plan.decode_tree(tree, want_lse=want_lse))
         plan.check()
-    assert none is None and torch.equal(out, again)
+    assert got[1][1] is None
+    for k, (out, lse) in enumerate(got):
+        tree.q.copy_(q0.roll(k, dims=0))
+        kw = oracle.tree_kwargs(tree.to("cpu"))
+        kw["chunk_node"] = kw.pop("leaf_node")
+        ref_o, ref_l = oracle.prefill(**kw)
+        PT.compare(tree, out, lse, ref_o, ref_l, None, f"{tree.name} call {k}")
 
 
 def test_prefill_e4m3_many_pairs():
