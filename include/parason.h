@@ -215,7 +215,8 @@ parason_status parason_attn_plan_shard_host(const parason_attn_config *cfg, int3
                                             int32_t world, int32_t num_sms, parason_plan *out);
 
 /* Device workspace (bytes) that parason_attn_decode needs for this plan:
- * the split partial results (o, m, l) of every work item.  0 for NULL. */
+ * the split partial results (o, m, l) of every work item.  0 for NULL, and for
+ * a prefill plan whose attention kernel writes the result itself (one launch). */
 size_t parason_plan_workspace_bytes(parason_plan plan);
 
 /*
@@ -242,13 +243,14 @@ size_t parason_plan_workspace_bytes(parason_plan plan);
  *            ignored otherwise (may be NULL)
  *   out      device, [num_leaves, H_q, head_dim], dtype of q, 16-byte
  *            aligned; or page-locked host memory the device can address
- *            (cudaHostAlloc / cudaHostRegister): the merge kernel then
- *            writes the result straight to the host
+ *            (cudaHostAlloc / cudaHostRegister): the plan's last kernel
+ *            then writes the result straight to the host
  *   lse      device (or such host memory) fp32 [num_leaves, H_q], or NULL.
  *            A branch whose whole path holds no token gets out = 0 and
  *            lse = -inf.
  *   workspace  device, at least parason_plan_workspace_bytes(plan) bytes,
- *            256-byte aligned; no contents are kept between calls.
+ *            256-byte aligned; no contents are kept between calls.  Ignored
+ *            (may be NULL) when that is 0.
  *
  * Slots of a node's last page past node_len are never read into the result,
  * whatever they hold (NaN included).

@@ -1732,7 +1732,7 @@ parason_status parason_attn_plan_shard_host(const parason_attn_config *cfg, int3
 }
 
 size_t parason_plan_workspace_bytes(parason_plan p) {
-    if (!p) return 0;
+    if (!p || p->direct) return 0;                  // direct: no partial rows
     const size_t o = align_up(static_cast<size_t>(p->num_slots) * p->cfg.head_dim * sizeof(float), kAlign);
     const size_t ml = align_up(static_cast<size_t>(p->num_slots) * sizeof(float2), kAlign);
     return o + ml;
@@ -1749,9 +1749,11 @@ parason_status parason_attn_decode(parason_plan p, const void *q, const void *k_
     if (!q || !out) return PARASON_EINVAL;
     const bool has_items = !p->items.empty();
     if (has_items) {
-        if (!k_pages || !v_pages || !workspace) return PARASON_EINVAL;
-        if (workspace_bytes < parason_plan_workspace_bytes(p)) return PARASON_EINVAL;
-        if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return PARASON_EINVAL;
+        if (!k_pages || !v_pages) return PARASON_EINVAL;
+        const size_t need = parason_plan_workspace_bytes(p);
+        if (need > 0 && (!workspace || workspace_bytes < need ||
+                         reinterpret_cast<uintptr_t>(workspace) % kAlign))
+            return PARASON_EINVAL;
         if (reinterpret_cast<uintptr_t>(k_pages) % 16 || reinterpret_cast<uintptr_t>(v_pages) % 16)
             return PARASON_EINVAL;
         if (p->cfg.mode == PARASON_FP8_E4M3_KV && (!k_scale || !v_scale)) return PARASON_EINVAL;

@@ -32,6 +32,7 @@ def test_short_chunks_are_cut(mode, h_q, h_kv, prefix, chunks, tokens, pairs):
         entries = plan.info()["num_wide_items"] // 2
         assert entries >= 2 * pairs and entries <= 4 * pairs
         assert plan.launches_per_decode() == 2
+        assert plan.workspace_bytes > 0
 
 
 @pytest.mark.parametrize("mode", ["bf16", "fp8"])
@@ -40,3 +41,4 @@ def test_whole_paths_stay_whole(mode, prefix, chunks, tokens):
     tree = _tree(mode, 32, 8, prefix, chunks, tokens)
     with Plan.for_prefill(tree, host_only=True, num_sms=SMS) as plan:
         assert plan.launches_per_decode() == 1
+        assert plan.workspace_bytes == 0        # the kernel writes the result: no partial rows

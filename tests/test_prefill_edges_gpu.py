@@ -101,6 +101,26 @@ def test_prefill_whole_paths_write_the_result(name, mode):
         PT.compare(tree, out, lse, ref_o, ref_l, None, f"{tree.name} call {k}")
 
 
+@pytest.mark.parametrize("mode", ["bf16", "fp8"])
+def test_prefill_whole_paths_need_no_workspace(mode):
+    tree = fork_tree(mode)
+    with Plan.for_prefill(tree) as plan:
+        assert plan.workspace_bytes == 0
+        ref = plan.decode_tree(tree)
+        out, lse = torch.full_like(tree.q, float("nan")), torch.full_like(ref[1], float("nan"))
+        scales = [None if s is None else s.data_ptr() for s in (tree.k_scale, tree.v_scale)]
+        st = _lib.load().parason_attn_decode(
+            plan.handle, tree.q.data_ptr(), tree.k_pages.data_ptr(), tree.v_pages.data_ptr(), *scales,
+            out.data_ptr(), lse.data_ptr(), None, 0, torch.cuda.current_stream().cuda_stream)
+        plan.check()
+        assert st == 0 and torch.equal(out, ref[0]) and torch.equal(lse, ref[1])
+        out.fill_(float("nan"))
+        plan.decode_no_alloc(tree.q, tree.k_pages, tree.v_pages, out, lse, k_scale=tree.k_scale,
+                             v_scale=tree.v_scale)
+        plan.check()
+        assert torch.equal(out, ref[0])
+
+
 def test_prefill_e4m3_many_pairs():
     """More than 4 tile pairs per SM with e4m3 KV: a run per node, not whole paths."""
     n = 4 * torch.cuda.get_device_properties(0).multi_processor_count // 16 + 2
