@@ -576,17 +576,17 @@ __device__ __forceinline__ void pages_step_t(const uint32_t *kbase, const uint32
     }
 }
 
-// Q fragments (A operand, row-major 16 x D) for tile rows rg*16 + {gid, gid+8}:
+// Q fragments (A operand, row-major 16 x D) for tile rows {gid, gid+8}:
 // bf16 as stored, or widened to f16 with d permuted as the e4m3 QK^T wants.
 template <int D, class KV>
-__device__ __forceinline__ void load_q_fragments(const AttnArgs &a, const WorkItem &it, int rg,
-                                                 int lane, uint32_t (&qa)[D / 16][4]) {
+__device__ __forceinline__ void load_q_fragments(const AttnArgs &a, const WorkItem &it, int lane,
+                                                 uint32_t (&qa)[D / 16][4]) {
     const int gid = lane >> 2, tig = lane & 3;
     const __nv_bfloat16 *qb = static_cast<const __nv_bfloat16 *>(a.q);
     const __nv_bfloat16 *qrow[2] = {nullptr, nullptr};
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int r = rg * 16 + gid + 8 * h;
+        const int r = gid + 8 * h;
         if (r < it.nrows) {
             const int nr = it.row0 + r;
             const int leaf = a.dfs_leaf[it.leaf_lo + nr / a.group];
@@ -623,12 +623,10 @@ __device__ __forceinline__ float2 item_scales(const AttnArgs &a, const WorkItem 
         return make_float2(a.scale_log2 * a.k_scale[it.kv_head], a.v_scale[it.kv_head]);
 }
 
-// A warp that owns rows rg*16 .. rg*16+15 of an item writes their partials
-// straight from registers.
+// A warp writes the partials of its item's up to 16 rows straight from registers.
 template <int D, class KV>
 __device__ __forceinline__ void store_warp_partials(const AttnArgs &a, const WorkItem &it,
-                                                    WarpState<D> &st, int rg, int lane,
-                                                    float o_scale) {
+                                                    WarpState<D> &st, int lane, float o_scale) {
     const int gid = lane >> 2, tig = lane & 3;
     st.l[0] += __shfl_xor_sync(0xffffffffu, st.l[0], 1);
     st.l[0] += __shfl_xor_sync(0xffffffffu, st.l[0], 2);
@@ -636,7 +634,7 @@ __device__ __forceinline__ void store_warp_partials(const AttnArgs &a, const Wor
     st.l[1] += __shfl_xor_sync(0xffffffffu, st.l[1], 2);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int r = rg * 16 + gid + 8 * h;
+        const int r = gid + 8 * h;
         if (r >= it.nrows) continue;
         const int64_t slot = static_cast<int64_t>(it.slot_base) + r;
         float *dst = a.part_o + slot * D;
@@ -799,10 +797,10 @@ __device__ void suffix_warp(const KvMaps &maps, const AttnArgs &a, uint32_t ring
         const WorkItem it = grab[k % kGrabSlots];
         const float2 scl = item_scales<KV>(a, it);
         if ((it.nrows > 4 || D == 64) && it.nrows <= 8) {
-            // one branch of 5 to 8 q heads: the transposed step (at head_dim 128
-            // tiles of up to 4 rows measured faster, at the tail, with the
-            // 16-row step; at head_dim 64, with two pages per update, slower:
-            // 16-branch step 23.3 -> 22.3 us)
+            // 5 to 8 rows, of one branch or several: the transposed step.  Up to 4
+            // rows take it at head_dim 64, where it runs two pages per update
+            // (16-branch step 23.3 -> 22.3 us); at head_dim 128 the 16-row step
+            // measured faster for them, at the tail
             uint32_t qb[D / 16][2];
             load_q_fragments_t<D, KV>(a, it, lane, qb);
             WarpStateT<D> st;
@@ -837,7 +835,7 @@ __device__ void suffix_warp(const KvMaps &maps, const AttnArgs &a, uint32_t ring
             continue;
         }
         uint32_t qa[D / 16][4];
-        load_q_fragments<D, KV>(a, it, 0, lane, qa);
+        load_q_fragments<D, KV>(a, it, lane, qa);
         WarpState<D> st;
         reset<D>(st);
         for (int pg = 0; pg < it.num_pages; ++pg, ++consumed) {
@@ -857,7 +855,7 @@ __device__ void suffix_warp(const KvMaps &maps, const AttnArgs &a, uint32_t ring
             issue_next();
         }
         if (!ok) break;
-        store_warp_partials<D, KV>(a, it, st, 0, lane, scl.y);
+        store_warp_partials<D, KV>(a, it, st, lane, scl.y);
     }
     if (!ok && lane == 0) dev::record_error(a.err, PARASON_ETIMEOUT, kSiteConsumerFull);
     // copies still in flight must land before the CTA's shared memory goes
@@ -884,10 +882,11 @@ __device__ void suffix_warp(const KvMaps &maps, const AttnArgs &a, uint32_t ring
 //               consecutive in the pool (the 5-D run maps), else one per
 //               page and column block; pages past the item's end are loaded
 //               from an out-of-range row, which TMA fills with zeros
-//   warp 9      S issuer (one lane): S = Q K^T (M 128, N 64, K 128) into
+//   warp 9      S issuer (the warp converged throughout, as elect.sync needs;
+//               one elected lane issues): S = Q K^T (M 128, N 64, K 128) into
 //               one of two TMEM buffers, once PV of the block two back has
 //               freed it; runs ahead across item boundaries
-//   warp 11     PV issuer (one lane): O += P V (M 128, N 128, K 64) into
+//   warp 11     PV issuer (likewise): O += P V (M 128, N 128, K 64) into
 //               the item's TMEM accumulator (two, alternating by item).
 //               A (Q or P) comes from TMEM, B (K or V) from shared memory.
 //               tcgen05.commit releases ring stages and signals completion.
@@ -1118,7 +1117,8 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
         // ------------------------------------------------------------ producer
         const bool skip_first = a.debug_flags & PARASON_DEBUG_SKIP_FIRST_LOAD;
         // bf16 KV: the tile's K and V go to L2 as evict-last (measured: the
-        // Llama-3-shape step 42.9 -> 41.4 us, the long-prefix one -1 us; no gain with e4m3 KV, which keeps the default)
+        // Llama-3-shape step 42.9 -> 41.4 us, the long-prefix one -1 us; no gain
+        // with e4m3 KV, which keeps the default)
         const uint64_t last_pol = dev::l2_evict_last_policy();
         // e4m3 blocks keep the default L2 policy (the per-page boxes use no hint)
         const uint64_t f8_pol = dev::l2_evict_normal_policy();
@@ -1619,9 +1619,10 @@ __device__ void prefix_cta_tc(const KvMaps *maps, const AttnArgs &a, uint8_t *sm
 //   warp 10     scheduler: pulls pairs and stages their metadata
 //   warp 8      producer: TMA of each block of the pair's pages, once, into
 //               a 4-stage ring
-//   warp 9      S issuer (one lane): S_t = Q_t K^T for t = A, B of a block,
+//   warp 9      S issuer (the warp converged, one elected lane issues): S_t =
+//               Q_t K^T for t = A, B of a block,
 //               A and B from shared memory
-//   warp 11     PV issuer (one lane): O_t += P_t V; the stage goes back to
+//   warp 11     PV issuer (likewise): O_t += P_t V; the stage goes back to
 //               the producer after the block's last PV
 //   warps 0-3   tile A: softmax (thread r owns row r, TMEM lane r), the next
 //               pair's Q rows into shared memory, then the row's (m, l) and O

@@ -609,7 +609,6 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
         int64_t pages;              // pages the run covers (from the node's first)
         int64_t node_pages = 0;     // pages of the node
         int64_t leaf_lo = 0;        // position of its first row's branch (query)
-        double cost_per_page;
         bool wide;
         bool causal = false;        // prefill: keys past the row's own token are masked
         int32_t span = -1;          // bf16 prefill: its page list in `spans`
@@ -695,8 +694,6 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
                             run.span = si;
                             run.leaf_lo = qbase[c];
                             run.wide = true;
-                            run.cost_per_page = wide_page_cost(cfg->head_dim, mode == PARASON_FP8_E4M3_KV);
-                            wide_cost += run.cost_per_page * static_cast<double>(run.pages);
                             runs.push_back(run);
                         }
                 }
@@ -722,8 +719,6 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
                                                : run.node_pages;
                         run.leaf_lo = qbase[c];
                         run.wide = true;
-                        run.cost_per_page = wide_page_cost(cfg->head_dim, mode == PARASON_FP8_E4M3_KV);
-                        wide_cost += run.cost_per_page * static_cast<double>(run.pages);
                         runs.push_back(run);
                     }
                 }
@@ -757,10 +752,8 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
                 run.node_pages = P;
                 run.leaf_lo = lo[n];
                 run.wide = wide;
-                run.cost_per_page =
-                    wide ? wide_page_cost(cfg->head_dim, mode == PARASON_FP8_E4M3_KV) : 1.0;
                 if (wide)
-                    wide_cost += run.cost_per_page *
+                    wide_cost += wide_page_cost(cfg->head_dim, mode == PARASON_FP8_E4M3_KV) *
                                  static_cast<double>(P + (mode == PARASON_FP8_E4M3_KV
                                                               ? std::min<int64_t>(kTcStartPagesE4m3, P / 3)
                                                               : 0));
