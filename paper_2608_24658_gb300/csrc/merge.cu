@@ -303,10 +303,17 @@ __global__ void __launch_bounds__(kMergeThreads)
 // LSE merge of two results: bound by HBM, so what counts is bytes in flight.  A
 // lane takes 16 bytes of a row (LPR lanes a row, all in one warp), and U rows
 // at once, every load requested before the first is used.  262,144 rows of
-// 128 bf16 (204 MB): 45.1 us with a warp per row and 8-byte loads, 33.2 us
-// with U = 4.  Few rows keep U = 1, which spreads them over more CTAs.
+// 128 bf16 (204 MB): 45.1 us with a warp per row and 8-byte loads, 37.0 with one
+// row a lane, 33.1 with kLseRows = 2, 33.3 with 4; of 128 fp32 59.9, 60.0 and 60.4
+// us (60,000 rows 16.6, 16.7 and 17.2: 4 was slower than a row per warp).
+//
+// Fewer rows keep U = 1, which spreads them over more CTAs: two rows a lane win
+// from about 608 CTAs of them on (4 per SM of a GB300).  In a graph, one against
+// two: 128 bf16, 8,000 rows 2.02 and 2.16 us, 16,000 2.78 and 2.77, 32,000 4.25
+// and 4.04; 128 fp32, 8,000 rows 2.26 and 2.50, 12,000 2.84 and 2.81.
 constexpr int kLseThreads = 256;
-constexpr int64_t kLseWideCtas = 608;                 // 4 per SM
+constexpr int kLseRows = 2;
+constexpr int64_t kLseWideCtas = 608;
 
 template <bool BF16>
 struct Vec16 {
@@ -439,11 +446,10 @@ template <int D, bool BF16>
 cudaError_t launch_lse(const void *o_a, const float *lse_a, const void *o_b, const float *lse_b,
                        void *o_out, float *lse_out, int64_t rows, cudaStream_t stream) {
     constexpr int kPass = kLseThreads / (D / Vec16<BF16>::N);
-    // U = 4 once that still gives every SM a few CTAs
-    const int u = rows >= int64_t{4} * kPass * kLseWideCtas ? 4 : 1;
+    const int u = rows >= int64_t{kLseRows} * kPass * kLseWideCtas ? kLseRows : 1;
     const int64_t blocks = (rows + int64_t{u} * kPass - 1) / (int64_t{u} * kPass);
     if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
-    const auto kernel = u == 4 ? lse_merge_kernel<D, BF16, 4> : lse_merge_kernel<D, BF16, 1>;
+    const auto kernel = u == kLseRows ? lse_merge_kernel<D, BF16, kLseRows> : lse_merge_kernel<D, BF16, 1>;
     kernel<<<static_cast<unsigned>(blocks), kLseThreads, 0, stream>>>(
         static_cast<const uint4 *>(o_a), lse_a, static_cast<const uint4 *>(o_b), lse_b,
         static_cast<uint4 *>(o_out), lse_out, rows);

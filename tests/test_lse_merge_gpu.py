@@ -1,6 +1,8 @@
 """parason_lse_merge around the edges of its launch: a row, a partial CTA, and
-both sides of the row count at which a lane takes four rows; in place too."""
+both sides of the row count at which a lane takes several rows; in place too."""
 import math
+import os
+import re
 
 import pytest
 import torch
@@ -9,13 +11,20 @@ from paper_2608_24658_gb300.api import lse_merge
 
 pytestmark = pytest.mark.gpu
 
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2608_24658_gb300", "csrc")
+
+
+def _constant(name):
+    with open(os.path.join(CSRC, "merge.cu")) as f:
+        return int(re.search(rf"constexpr \w+ {name} = (\d+);", f.read()).group(1))
+
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("in_place", [False, True])
 def test_lse_merge_row_edges(d, dtype, in_place):
-    rows_per_pass = 256 * 16 // (d * dtype.itemsize)
-    wide = 4 * 608 * rows_per_pass
+    rows_per_pass = _constant("kLseThreads") * 16 // (d * dtype.itemsize)
+    wide = _constant("kLseRows") * _constant("kLseWideCtas") * rows_per_pass
     for rows in (1, 3, rows_per_pass, rows_per_pass + 1, wide - 1, wide, wide + 5):
         gen = torch.Generator(device="cuda")
         gen.manual_seed(rows)
