@@ -253,7 +253,10 @@ size_t parason_plan_workspace_bytes(parason_plan plan);
  *            (may be NULL) when that is 0.
  *
  * Slots of a node's last page past node_len are never read into the result,
- * whatever they hold (NaN included).
+ * whatever they hold (NaN included).  A NaN or infinity in V of a token the
+ * node does hold reaches every query that sees the token; in a prefill it may
+ * also reach up to 2 floor(128 / g) + 14 queries before the token in its chunk
+ * (g = H_q / H_kv), whose weight for it is 0: they share its tiles and pages.
  *
  * With e4m3 KV the kernels multiply q by the widened keys and values in f16
  * (f16 holds every e4m3 value exactly): q is narrowed from bf16 to f16,

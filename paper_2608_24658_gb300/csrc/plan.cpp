@@ -7,7 +7,8 @@
 //
 //  * every node n that some branch reads is processed once per kv head, with
 //    all R_n = (#branches under n) * g query rows stacked into tiles of up to
-//    64 rows, so the node's KV is read from HBM once for all of them;
+//    128 rows (16 in fp32 mode and the suffix pass), so the node's KV is read
+//    from HBM once for all of them;
 //  * long nodes are cut into chunks of whole pages (split-K) so that the
 //    grid fills the GPU; each (node, chunk, kv head) has R_n partial slots;
 //  * branch b's result is the log-sum-exp merge of the partial slots of every
@@ -31,9 +32,8 @@ using parason::WorkItem;
 namespace {
 
 constexpr int kNarrowRows = 16;         // nodes with at most this many rows: suffix pass
-// autonomous warps per suffix-pass CTA (the kernel's count for the KV format)
-// (the kernel's count for the KV format: 6 deeper warps for bf16 at head_dim
-// 128 with g <= 4, where they are latency-bound)
+// autonomous warps per suffix-pass CTA (the kernel's count for the KV format: 6
+// deeper warps for bf16 at head_dim 128 with g <= 4, where they are latency-bound)
 int32_t narrow_warps(int32_t mode, int32_t head_dim, int32_t g) {
     if (mode == PARASON_FP8_E4M3_KV) return 12;
     return (mode == PARASON_BF16 && head_dim == 128 && g <= 4) ? 6 : 8;
@@ -84,7 +84,10 @@ constexpr int kPieceCounts = 8;
 // With e4m3 KV a prefill of up to this many pairs per SM reads whole paths
 // (one list of pages per pair and kv head, as with bf16 KV), of more a run per
 // node: join prefill 796 -> 664 us, fork 78.9 -> 54.2, 30 chunks of 2 to 5 tokens
-// with 16 kv heads (3.2 pairs an SM) 42.2 -> 25.2.
+// with 16 kv heads (3.2 pairs an SM) 42.2 -> 25.2.  The line is where the
+// measurements ended when it was drawn; it is no crossing: at 5 to 27 pairs an SM
+// whole paths are ahead as well, by 1% to 96% on 56 of 57 prefills, most over
+// paths of many nodes.
 constexpr int64_t kListPairsE4m3 = 4;
 constexpr int kPrefillBlockPages = parason::kPrefillBoxPages;   // a prefill tile's blocks
 // Suffix pieces: at most about kNarrowPiecesPerWarp per warp of the launch (and
@@ -95,18 +98,16 @@ constexpr int kPrefillBlockPages = parason::kPrefillBoxPages;   // a prefill til
 // (bf16 KV: HBM is then no longer full; e4m3 KV keeps them closer to their own
 // pace).  What decides is how the nodes' lengths divide: on 64 branches of 16
 // heads with e4m3 KV pieces of 41, 52, 65 and 83 pages took 131, 149, 128 and
-// 141 us.  Start and share were fitted to 16 trees at 10 to 13 lengths each;
-// the lengths chosen are within 2% (e4m3) and 1% (bf16) of the best of them, a
-// fixed 2 and 2.5 pieces per warp within 12% and 4%.
-// Against those: 16 branches 31.5 -> 30.2 us, two-level tree 69.3 -> 67.2, 4
-// requests x 32 branches at head_dim 64 42.0 -> 41.0; e4m3 KV 8k prefix and 64
-// branches 66.7 -> 63.4, 9 requests of 47 branches 128 -> 110 (slower: 64 branches
-// of a 16k prefix at head_dim 64 87.5 -> 90.2).  The choice takes no longer than
-// the items it saves (a plan of 1024 branches 8.4 -> 8.1 ms).
+// 141 us.  Start and share were fitted to 16 trees.  On 220 others at up to 11 lengths each the lengths chosen are, in the
+// mean and at worst, 1.2% and 6.5% off the best of them (bf16 KV, head_dim 128),
+// 2.3% and 10% (head_dim 64), 2.2% and 19% (e4m3 KV); a fixed 2.5 pieces per warp
+// 2.3% and 10%, 5.6% and 16%, 10.5% and 25%; one piece per warp 6%, 10% and 9%.
+// The choice takes no longer than the items it saves (a plan of 1024 branches
+// 8.4 -> 8.1 ms).
 constexpr double kNarrowPiecesPerWarp = 2.5;
 constexpr int64_t kNarrowStartPages = 2, kNarrowStartPagesE4m3 = 8;
 constexpr double kNarrowFullShare = 0.5, kNarrowFullShareE4m3 = 0.8;
-constexpr int kNarrowLengths = 10;         // lengths tried
+constexpr int kNarrowLengths = 10;         // steps from 2.5 pieces per warp to one: a length each
 constexpr int64_t kNarrowTimeMax = 1 << 14;   // pages of a warp, where lengths matter little
 constexpr double kWideProvision = 1.15;   // prefix CTAs relative to the cost model
 // A prefix tile's start and its O take a CTA 3.5 us (head_dim 64) to 5 us, which
@@ -149,7 +150,11 @@ constexpr int kFp32ChunkPages = 32;
 // launches a share of their time.  Same-box A/B: 16-branch step 34.0 -> 31.2
 // us, two-level 74.2 -> 69.3, 1.5 GB of bf16 KV 243 -> 230, 5.7 GB 834 -> 836;
 // e4m3 KV 0.23 GB 87 -> 84 us, 0.74 GB level, 2.9 GB 517 -> 529; fork prefill
-// (132 pages a CTA) 41.8 -> 39.9 us, join prefill (2150) 524 -> 538.
+// (132 pages a CTA) 41.8 -> 39.9 us, join prefill (2150) 524 -> 538.  Between
+// those, chunks of 64 and of 1024 tokens under 1k to 16k prefixes: bf16 KV
+// 7% to 2% faster early at 43 to 250 pages a CTA, 2% to 1% at 430 to 900, level
+// from 1000 on; e4m3 KV 5% to 2% faster for 16 chunks of 64 tokens and up to 6%
+// slower for one of 1024, at any count.
 constexpr int64_t kEarlyKvBytes = int64_t{2} << 30, kEarlyKvBytesE4m3 = int64_t{3} << 28;
 constexpr int64_t kEarlyPrefillPages = 256;    // a CTA's share
 constexpr int kFp32MinPages = 4;
@@ -611,15 +616,17 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
         int64_t leaf_lo = 0;        // position of its first row's branch (query)
         bool wide;
         bool causal = false;        // prefill: keys past the row's own token are masked
-        int32_t span = -1;          // bf16 prefill: its page list in `spans`
+        int32_t span = -1;          // prefill of whole paths: its page list in `spans`
     };
-    // A bf16 prefill run reads its chunk's whole path in one list of pages:
-    // every page of every non-empty ancestor, root first, then the chunk's
-    // own pages up to the tile pair's last token.  Its pieces cross node
-    // boundaries, so that each query row has a partial per piece of its path
-    // rather than one per node.  An ancestor that ends inside a page is
-    // followed by padding pages (zero-filled by TMA) up to the next 64-token
-    // block, so that the keys no token stands for always end a block.
+    // A prefill run of whole paths (`lists`: bf16 KV, and e4m3 KV up to
+    // kListPairsE4m3) reads its chunk's path in one list of pages: every page of
+    // every non-empty ancestor, root first, then the chunk's own pages up to the
+    // tile pair's last token.  Its pieces cross node boundaries, so that each
+    // query row has a partial per piece of its path rather than one per node.
+    // An ancestor that ends inside a page is followed by padding pages
+    // (zero-filled by TMA) up to the next 64-token half of a block, so that the
+    // keys no token stands for always end a half (the kernel keeps a count of
+    // valid keys per half).
     struct Span {
         std::vector<int32_t> pos;     // position in page_ids of each page, -1: padding
         std::vector<int32_t> valid;   // valid tokens of each page

@@ -45,11 +45,10 @@
 // the launch holds).
 //
 // Measured (32 q / 8 kv heads, attention kernel): join, 1024 queries over 41k
-// keys, 486 us of 356 us of arithmetic at 1.9 PFLOP/s, where the decode
-// kernel's pair tile took 583 us; with e4m3 KV 730 us against 970 us with a run
-// per node (797 us a pass, 663 with whole paths); fork, 16 x
-// 64 queries over 2112 keys, 45 us and no merge against 53 us and a merge.  A
-// pair of blocks takes about 3400 cycles against 2048 of tensor work: a tile's
+// keys, 486 us of 348 us of arithmetic at 1.95 PFLOP/s, where the decode
+// kernel's pair tile took 583 us; with e4m3 KV 654 us (whole paths) against 970;
+// fork, 16 x 64 queries over 2112 keys, a pass of 39 us without a merge against 59
+// with one.  A pair of blocks takes about 3400 cycles against 2048 of tensor work: a tile's
 // chain is 300 cycles to read S, 400 for the maxima, 1100 for the
 // exponentials, then 768 of its own PV half and S.  Tried and slower: an issuer
 // per tile (both tiles fall into step, 555 -> 727 us), the first half
