@@ -81,13 +81,15 @@ constexpr PrefillCost kPrefillE4m3 = {1.35, 0.85, 36.0, 8.0};
 constexpr double kEntryRowPages = 0.01, kPartialRowPages = 0.12, kOutRowPages = 0.15;
 constexpr double kPullPages = 7.0, kPullLeadBlocks = 6.0;
 constexpr int kPieceCounts = 8;
-// With e4m3 KV a prefill of up to this many pairs per SM reads whole paths
-// (one list of pages per pair and kv head, as with bf16 KV), of more a run per
-// node: join prefill 796 -> 664 us, fork 78.9 -> 54.2, 30 chunks of 2 to 5 tokens
-// with 16 kv heads (3.2 pairs an SM) 42.2 -> 25.2.  The line is where the
-// measurements ended when it was drawn; it is no crossing: at 5 to 27 pairs an SM
-// whole paths are ahead as well, by 1% to 96% on 56 of 57 prefills, most over
-// paths of many nodes.
+// With e4m3 KV a prefill reads whole paths (one list of pages per pair and kv
+// head, as with bf16 KV) on a device of kListSms SMs or more: join prefill 796 ->
+// 664 us, fork 78.9 -> 54.2, 30 chunks of 2 to 5 tokens with 16 kv heads 42.2 ->
+// 25.2; of 57 prefills of 5 to 27 pairs an SM 56 by 1% to 96%, one 1% slower.  (A run
+// per node, as those had, took 19 of 60 of them 2% to 45% longer than the decode
+// kernel's tile: 60 chunks of 5 tokens over 9 nodes, 16 kv heads, 529 us then, 768
+// so, 518 with whole paths.)  Smaller partitions were not measured: there up to
+// kListPairsE4m3 pairs per SM read whole paths, more a run per node.
+constexpr int32_t kListSms = 32;
 constexpr int64_t kListPairsE4m3 = 4;
 constexpr int kPrefillBlockPages = parason::kPrefillBoxPages;   // a prefill tile's blocks
 // Suffix pieces: at most about kNarrowPiecesPerWarp per warp of the launch (and
@@ -618,8 +620,8 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
         bool causal = false;        // prefill: keys past the row's own token are masked
         int32_t span = -1;          // prefill of whole paths: its page list in `spans`
     };
-    // A prefill run of whole paths (`lists`: bf16 KV, and e4m3 KV up to
-    // kListPairsE4m3) reads its chunk's path in one list of pages: every page of
+    // A prefill run of whole paths (`lists`; e4m3 KV on a small partition may have
+    // runs per node) reads its chunk's path in one list of pages: every page of
     // every non-empty ancestor, root first, then the chunk's own pages up to the
     // tile pair's last token.  Its pieces cross node boundaries, so that each
     // query row has a partial per piece of its path rather than one per node.
@@ -648,7 +650,8 @@ parason_status build_host(parason_plan_s *p, const parason_attn_config *cfg, int
             pairs += H_kv * ((R + 2 * rt - 1) / (2 * rt));
         }
         lists = cfg->head_dim == 128 &&
-                (mode == PARASON_BF16 || pairs <= kListPairsE4m3 * static_cast<int64_t>(p->num_sms));
+                (mode == PARASON_BF16 || p->num_sms >= kListSms ||
+                 pairs <= kListPairsE4m3 * static_cast<int64_t>(p->num_sms));
         // chunk c: rows (token t, q head r) = t * g + r of every kv head, in
         // tiles that run in pairs; each pair reads every ancestor in full and
         // its own node up to the pair's last token

@@ -122,7 +122,7 @@ def test_prefill_whole_paths_need_no_workspace(mode):
 
 
 def test_prefill_e4m3_many_pairs():
-    """More than 4 tile pairs per SM with e4m3 KV: a run per node, not whole paths."""
+    """More than 4 tile pairs per SM with e4m3 KV: several whole paths a CTA, and a merge."""
     n = 4 * torch.cuda.get_device_properties(0).multi_processor_count // 16 + 2
     tree = W.build_prefill("many", [-1, 0] + [1] * n, [70, 9] + [1 + k % 3 for k in range(n)],
                            list(range(2, 2 + n)), num_q_heads=16, num_kv_heads=16, head_dim=128,

@@ -28,3 +28,17 @@ def test_e4m3_list_rule(chunks, lists):
         verify_prefill_plan(t, plan)
         rng = plan.export(_lib.TABLE_MERGE_RANGES)
         assert ((rng[:, 1] - rng[:, 0] == 1).all()) == lists
+
+
+@pytest.mark.parametrize("sms,lists", [(31, False), (32, True), (152, True)])
+def test_e4m3_many_pairs_read_whole_paths(sms, lists):
+    """More than 4 pairs an SM: whole paths but on a small partition."""
+    n = 5 * 152 // 4
+    t = W.build_prefill("many", [-1, 0] + [1] * n, [70, 9] + [1 + k % 3 for k in range(n)],
+                        list(range(2, 2 + n)), num_q_heads=4, num_kv_heads=4, head_dim=128,
+                        mode="fp8", values=False)
+    with Plan.for_prefill(t, host_only=True, num_sms=sms) as plan:
+        verify_prefill_plan(t, plan)
+        assert plan.info()["num_wide_items"] // 2 >= 5 * sms
+        rows = plan.export(_lib.TABLE_STREAM_ROWS)
+        assert (rows & 15).any() == lists          # a node's end inside an item
