@@ -478,7 +478,7 @@ parason_status parason_plan_get_info(parason_plan plan, parason_plan_info *info)
  *                            page-count entries from there)
  *   PARASON_TABLE_STREAM_ROWS int32 [num_stream_rows]: the TMA row
  *                            (page * H_kv + kv head) * 16 of every item page;
- *                            in a bf16 prefill piece over several nodes of a
+ *                            in a prefill piece over several nodes of a
  *                            path, a page that ends a node before the item's
  *                            last page adds 16 - its valid tokens (1..15),
  *                            and is followed up to the next 4-page block by
