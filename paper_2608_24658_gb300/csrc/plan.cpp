@@ -100,10 +100,12 @@ constexpr int kPrefillBlockPages = parason::kPrefillBoxPages;   // a prefill til
 // (bf16 KV: HBM is then no longer full; e4m3 KV keeps them closer to their own
 // pace).  What decides is how the nodes' lengths divide: on 64 branches of 16
 // heads with e4m3 KV pieces of 41, 52, 65 and 83 pages took 131, 149, 128 and
-// 141 us.  Start and share were fitted to 16 trees.  On 220 others at up to 11 lengths each the lengths chosen are, in the
-// mean and at worst, 1.2% and 6.5% off the best of them (bf16 KV, head_dim 128),
-// 2.3% and 10% (head_dim 64), 2.2% and 19% (e4m3 KV); a fixed 2.5 pieces per warp
-// 2.3% and 10%, 5.6% and 16%, 10.5% and 25%; one piece per warp 6%, 10% and 9%.
+// 141 us.  Start and share were fitted to 16 trees.  On 220 others at up to 11
+// lengths each the lengths chosen are, in the mean and at worst, 1.2% and 6.5% off
+// the best of them (bf16 KV, head_dim 128), 2.3% and 10% (head_dim 64), 2.2% and
+// 19% (e4m3 KV); a fixed 2.5 pieces per warp 2.3% and 10%, 5.6% and 16%, 10.5% and
+// 25%; one piece per warp 6%, 10% and 9%.  20 of the 220 are slower than with 2.5
+// by 2% to 9%.
 // The choice takes no longer than the items it saves (a plan of 1024 branches
 // 8.4 -> 8.1 ms).
 constexpr double kNarrowPiecesPerWarp = 2.5;
